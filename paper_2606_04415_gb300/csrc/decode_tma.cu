@@ -1,6 +1,10 @@
 // Decode split-KV attention fed by TMA through an mbarrier ring
-// (Hkv = 4 kv heads, d = 64 or 128, G <= 8 query heads per kv head, block
-// size a multiple of 16).
+// (d = 64 or 128, G <= 8 query heads per kv head, block size a multiple of
+// 16). An item covers up to four kv heads of its keys; with more than four,
+// the heads go in groups of four, each an item of its own. (For 32 query and
+// 8 kv heads, a 1024-token chunk beside 64 decodes: 140.0 us with the per-head
+// cp.async kernel ahead of the prefill, whose decode streams 2.8 TB/s; 100.4
+// us with this one beside the prefill.)
 //
 // Decode is bound by KV-cache reads (Sec. 1, Sec. 3.3, Fig. 2). The kernel is
 // kept small -- five warps, at most 128 registers a thread, 64 KB of shared
@@ -14,9 +18,10 @@
 //     block-table row and first four block ids, so that a CTA issues its
 //     first copies one load after it starts. (Taking two items ahead left
 //     CTAs idle when items were few: the first CTAs reserved them all.)
-//   * A 2-stage ring of 16-key stages holds K and V of all four kv heads. A
+//   * A 2-stage ring of 16-key stages holds K and V of the item's kv heads. A
 //     producer warp issues the TMA copies (four boxes of 16 slots x 4 heads x
-//     64 columns for d = 128) as soon as a stage is free; issuing them from a
+//     64 columns for d = 128; heads past the last are filled with zeros and
+//     their warps only release the stages) as soon as a stage is free; issuing them from a
 //     compute warp cost that warp about as much as its arithmetic. The tensor map
 //     lists the slot dimension before the kv-head dimension, so a box lands
 //     head-major (16 consecutive slots of one head form 16 rows) and the
@@ -42,7 +47,7 @@
 namespace fnpu {
 namespace {
 
-constexpr int kHkv = 4;
+constexpr int kHkv = 4;          // kv heads per item
 constexpr int kKeys = 16;        // keys per stage
 constexpr int kStages = 2;
 constexpr int kWarps = 4;        // compute warps, one per kv head
@@ -77,6 +82,7 @@ struct DtGeo {
     int kb, ke;     // keys [kb, ke)
     int split, ns, part_base, group;
     int b0, b1, b2, b3;  // ids of the item's first four blocks
+    int head0;      // first kv head
 };
 
 template <int D>
@@ -102,7 +108,9 @@ __device__ __forceinline__ int load_blk_lane(const AttnParams &p, const DtGeo &g
     return lane < nblk ? __ldg(p.block_table + static_cast<int64_t>(g.bt_row) * p.bt_stride + b0 + lane) : 0;
 }
 
-template <int D>
+// kRagged: the kv heads are no multiple of four, so that a warp of the last
+// group may have none (the checks cost a small step 7% where they are not needed)
+template <int D, bool kRagged>
 __global__ void __launch_bounds__(kThreads, 3)
     decode_tma_kernel(const AttnParams p, const __grid_constant__ DtMaps maps) {
     using Cfg = DtCfg<D>;
@@ -159,10 +167,14 @@ __global__ void __launch_bounds__(kThreads, 3)
         g.ns = it.num_splits;
         g.part_base = it.part_base;
         g.group = it.group;
+        g.head0 = it.kvh;
         return g;
     };
 
-    const int head = warp;
+    const uint32_t stage_bytes =
+        kRagged && p.num_kv_heads < kHkv ? Cfg::kStageBytes / kHkv * p.num_kv_heads : Cfg::kStageBytes;
+    const int wh = warp;  // kv head of this warp within the item's
+    auto has_head = [&](const DtGeo &g) { return !kRagged || g.head0 + wh < p.num_kv_heads; };
     const int g8 = lane >> 2, c = lane & 3;
     const int lj = lane >> 3, lr = lane & 7;
     const int G = p.group;
@@ -184,11 +196,11 @@ __global__ void __launch_bounds__(kThreads, 3)
             if (rel >= 32) blk = __ldg(p.block_table + static_cast<int64_t>(g.bt_row) * p.bt_stride + key0 / bs);
         }
         const uint32_t sK = s_base + st * Cfg::kStageBytes, sV = sK + Cfg::kTileBytes;
-        tc::mbar_arrive_expect_tx_warp(FULL(st), Cfg::kStageBytes);
+        tc::mbar_arrive_expect_tx_warp(FULL(st), stage_bytes);
 #pragma unroll
         for (int h = 0; h < D / 64; ++h) {
-            tc::tma_load_4d_warp(sK + h * kHalfBytes, &maps.k, FULL(st), h * 64, key0 % bs, 0, blk);
-            tc::tma_load_4d_warp(sV + h * kHalfBytes, &maps.v, FULL(st), h * 64, key0 % bs, 0, blk);
+            tc::tma_load_4d_warp(sK + h * kHalfBytes, &maps.k, FULL(st), h * 64, key0 % bs, g.head0, blk);
+            tc::tma_load_4d_warp(sV + h * kHalfBytes, &maps.v, FULL(st), h * 64, key0 % bs, g.head0, blk);
         }
         return true;
     };
@@ -245,7 +257,7 @@ __global__ void __launch_bounds__(kThreads, 3)
             cur = geo_of(p.ditems[idx]);
         }
         uint32_t qb[D / 16][2];
-        load_q<D>(p, cur.t, head, g8, c, qb);
+        if (has_head(cur)) load_q<D>(p, cur.t, cur.head0 + wh, g8, c, qb);
         bool ok = true;
         int g = 0;  // ring position of the current item's first stage
         for (int k = 0; ok; ++k) {
@@ -274,12 +286,13 @@ __global__ void __launch_bounds__(kThreads, 3)
                 const uint32_t sK = s_base + st * Cfg::kStageBytes, sV = sK + Cfg::kTileBytes;
                 const int nv = nkeys - i * kKeys;  // valid keys in this stage (>= 1)
                 const bool tail = nv < kKeys;
+                if (has_head(cur)) {  // (warp-uniform; else the warp only releases the stage)
                 if (tail) {  // zero this head's V rows past the item's keys
                     for (int e = lane; e < (kKeys - nv) * 8 * (D / 64); e += 32) {
                         const int hh = e / ((kKeys - nv) * 8), rem = e % ((kKeys - nv) * 8);
                         const int sl = nv + rem / 8, ch = rem % 8;
                         *reinterpret_cast<uint4 *>(smem + st * Cfg::kStageBytes + Cfg::kTileBytes + hh * kHalfBytes +
-                                                   (head * kKeys + sl) * 128 + ch * 16) = make_uint4(0u, 0u, 0u, 0u);
+                                                   (wh * kKeys + sl) * 128 + ch * 16) = make_uint4(0u, 0u, 0u, 0u);
                     }
                     __syncwarp();
                 }
@@ -287,7 +300,7 @@ __global__ void __launch_bounds__(kThreads, 3)
 #pragma unroll
                 for (int kk = 0; kk < D / 16; ++kk) {
                     uint32_t a0, a1, a2, a3;
-                    ldmatrix_x4(a0, a1, a2, a3, sK + dt_off(lr + 8 * (lj & 1), head, 2 * kk + (lj >> 1)));
+                    ldmatrix_x4(a0, a1, a2, a3, sK + dt_off(lr + 8 * (lj & 1), wh, 2 * kk + (lj >> 1)));
                     mma_bf16_16816(s, a0, a1, a2, a3, qb[kk][0], qb[kk][1]);
                 }
                 const bool v0 = g8 < nv, v1 = g8 + 8 < nv;
@@ -317,17 +330,18 @@ __global__ void __launch_bounds__(kThreads, 3)
 #pragma unroll
                 for (int mt = 0; mt < D / 16; ++mt) {
                     uint32_t a0, a1, a2, a3;
-                    ldmatrix_x4_trans(a0, a1, a2, a3, sV + dt_off(lr + 8 * (lj >> 1), head, 2 * mt + (lj & 1)));
+                    ldmatrix_x4_trans(a0, a1, a2, a3, sV + dt_off(lr + 8 * (lj >> 1), wh, 2 * mt + (lj & 1)));
                     mma_bf16_16816(o[mt], a0, a1, a2, a3, pb0, pb1);
                 }
                 if (tail) tc::fence_proxy_async_smem();  // order the zeroing before the next TMA write
+                }
                 __syncwarp();
                 tc::mbar_arrive_warp(EMPTY(st));
                 // the next item's query: a stage after its descriptor (at once for
                 // a short item)
                 if (has_next && i == (spub + 1 < ntiles ? spub + 1 : spub)) {
                     nxt = geo_of(nit);
-                    load_q<D>(p, nxt.t, head, g8, c, qn);
+                    if (has_head(nxt)) load_q<D>(p, nxt.t, nxt.head0 + wh, g8, c, qn);
                 }
             }
             if (!ok) break;
@@ -338,7 +352,9 @@ __global__ void __launch_bounds__(kThreads, 3)
             l1 += __shfl_xor_sync(0xffffffffu, l1, 8);
             l1 += __shfl_xor_sync(0xffffffffu, l1, 16);
             const float inv0 = 1.f / l0, inv1 = 1.f / l1;
-            const int h0 = 2 * c, h1 = 2 * c + 1;  // this lane's query heads within the group
+            const int head = cur.head0 + wh;  // kv head
+            // this lane's query heads within the group (none for a warp without a kv head)
+            const int h0 = has_head(cur) ? 2 * c : G, h1 = has_head(cur) ? 2 * c + 1 : G;
             if (cur.ns == 1) {
 #pragma unroll
                 for (int mt = 0; mt < D / 16; ++mt) {
@@ -481,8 +497,8 @@ __global__ void __launch_bounds__(32 * kMergeWarps) split_merge_kernel(const Att
 }
 
 // 4-D map over a paged cache [num_blocks, bs, Hkv, d] with the slot dimension
-// listed before the kv-head dimension: a box (64 columns, 16 slots, Hkv heads,
-// 1 block) lands in shared memory head-major.
+// listed before the kv-head dimension: a box (64 columns, 16 slots, up to four
+// kv heads, 1 block) lands in shared memory head-major.
 bool encode_slot_major_map(CUtensorMap *m, const void *base, int d, int hkv, int bs, int nblocks) {
     EncodeTiledFn enc = tensor_map_encoder();
     if (!enc) return false;
@@ -490,42 +506,45 @@ bool encode_slot_major_map(CUtensorMap *m, const void *base, int d, int hkv, int
                           static_cast<cuuint64_t>(nblocks)};
     cuuint64_t strides[3] = {static_cast<cuuint64_t>(hkv) * d * 2, static_cast<cuuint64_t>(d) * 2,
                              static_cast<cuuint64_t>(bs) * hkv * d * 2};
-    cuuint32_t box[4] = {64, static_cast<cuuint32_t>(kKeys), static_cast<cuuint32_t>(hkv), 1};
+    cuuint32_t box[4] = {64, static_cast<cuuint32_t>(kKeys), static_cast<cuuint32_t>(hkv < kHkv ? hkv : kHkv), 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D>
+template <int D, bool kRagged>
 int launch_dt(const AttnParams &p, cudaStream_t st, int max_ctas) {
     using Cfg = DtCfg<D>;
+    auto kernel = decode_tma_kernel<D, kRagged>;
     DtMaps maps;
     if (!encode_slot_major_map(&maps.k, p.k_cache, D, p.num_kv_heads, p.block_size, p.num_blocks) ||
         !encode_slot_major_map(&maps.v, p.v_cache, D, p.num_kv_heads, p.block_size, p.num_blocks))
         return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled (decode)");
-    FNPU_CUDA_TRY(cudaFuncSetAttribute(decode_tma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       Cfg::kSmemBytes));
-    FNPU_CUDA_TRY(cudaFuncSetAttribute(decode_tma_kernel<D>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    FNPU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
+    FNPU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        cudaSharedmemCarveoutMaxShared));
     const int grid = p.num_ditems < max_ctas ? p.num_ditems : max_ctas;
-    FNPU_CUDA_TRY(launch_ex(decode_tma_kernel<D>, grid, kThreads, Cfg::kSmemBytes, st, false, nullptr, p, maps));
+    FNPU_CUDA_TRY(launch_ex(kernel, grid, kThreads, Cfg::kSmemBytes, st, false, nullptr, p, maps));
     return FNPU_OK;
 }
 
 }  // namespace
 
 bool decode_tma_supported(int d_qk, int d_v, int hkv, int group, int block_size) {
-    return d_qk == d_v && (d_qk == 64 || d_qk == 128) && hkv == kHkv && group <= 8 && block_size % kKeys == 0;
+    (void)hkv;
+    return d_qk == d_v && (d_qk == 64 || d_qk == 128) && group <= 8 && block_size % kKeys == 0;
 }
+
+int decode_tma_heads_per_item() { return kHkv; }
 
 int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas) {
     if (p.num_ditems == 0) return FNPU_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int rc = FNPU_EUNSUPPORTED;
     switch (p.head_dim_qk) {
-        case 64: rc = launch_dt<64>(p, st, max_ctas); break;
-        case 128: rc = launch_dt<128>(p, st, max_ctas); break;
+        case 64: rc = p.num_kv_heads % kHkv ? launch_dt<64, true>(p, st, max_ctas) : launch_dt<64, false>(p, st, max_ctas); break;
+        case 128: rc = p.num_kv_heads % kHkv ? launch_dt<128, true>(p, st, max_ctas) : launch_dt<128, false>(p, st, max_ctas); break;
         default: break;
     }
     if (rc != FNPU_OK) return rc;

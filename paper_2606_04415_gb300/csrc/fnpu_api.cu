@@ -698,11 +698,13 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
             it.blk[i] = block_table[static_cast<int64_t>(s) * block_table_stride + kb / bs + i];
         return it;
     };
+    // items per key range: one per group of kv heads (TMA kernel), one per kv head
+    const int32_t hpi = pl->use_dt ? decode_tma_heads_per_item() : 1;
+    const int32_t hgroups = (desc->num_kv_heads + hpi - 1) / hpi;
     int64_t dec_keys = 0;
     for (int32_t s = 0; s < num_seqs; ++s)
-        if (decode_queue(s))
-            dec_keys += static_cast<int64_t>(context_len[s]) * (pl->use_dt ? 1 : desc->num_kv_heads);
-    int32_t split = o.decode_split_keys;
+        if (decode_queue(s)) dec_keys += static_cast<int64_t>(context_len[s]) * hgroups;
+    int32_t split = std::min(o.decode_split_keys, 1 << 30);  // (room to round up)
     if (split == 0) {
         const int64_t target = (pl->use_dt ? 2LL : 6LL) * sms;
         int64_t sk = (dec_keys + target - 1) / std::max<int64_t>(target, 1);
@@ -780,9 +782,10 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
                 }
             }
         } else if (decode_queue(s) && pl->use_dt) {
-            // items over all kv heads; a split sequence is merged by the merge
-            // kernel (at most 256 splits: its scratch grows with them)
-            const int32_t sk = std::max(split, (c + 256 * 64 - 1) / (256 * 64) * 64);
+            // items over groups of kv heads, cut at whole 16-key stages; a
+            // split sequence is merged by the merge kernel (at most 256
+            // splits: its scratch grows with them)
+            const int32_t sk = std::max((split + 15) / 16 * 16, (c + 256 * 64 - 1) / (256 * 64) * 64);
             const int32_t ns = (c + sk - 1) / sk;
             const int32_t base = ns > 1 ? parts : 0;
             if (ns > 1) {
@@ -791,7 +794,8 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
             }
             for (int32_t sp = 0; sp < ns; ++sp) {
                 const int32_t kb = sp * sk, ke = std::min(c, kb + sk);
-                ditems.push_back(decode_item(s, 0, kb, ke, sp, ns, base, 0));
+                for (int32_t hg = 0; hg < hgroups; ++hg)
+                    ditems.push_back(decode_item(s, hg * hpi, kb, ke, sp, ns, base, 0));
             }
         } else if (decode_queue(s)) {
             const int32_t ns = (c + split - 1) / split;
@@ -832,17 +836,29 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
     // CTAs hold the rest
     pl->coloc = pl->use_tc && pl->use_dt && !tc_units.empty() && !ditems.empty() &&
                 !(o.flags & FNPU_PLAN_SEPARATE_LAUNCHES);
+    const double tile_scale = (desc->head_dim_qk + desc->head_dim_v) / 256.0;  // relative to d = 128
+    if (pl->coloc && desc->num_kv_heads != 4 && o.decode_share_pct == 0 && !(o.flags & FNPU_PLAN_GREEN_CONTEXTS)) {
+        // A prefill of one or two short tiles is over before the fork, the
+        // join and the wait for its start are paid for: with a chunk of 128
+        // tokens, d = 64 and no prefix (2.3 us by the model) a re-planned
+        // step takes 28.6 us with the phases in turn and 42.6 co-located;
+        // from about 5 us on co-location wins (chunks of 32 to 512 tokens:
+        // 26.6 us against 28.7, 32.9 against 39.6, 35.6 against 43.1). Four kv
+        // heads co-locate always: such plans report phase times.
+        int32_t longest = 0;
+        for (const TcUnit &u : tc_units) longest = std::max(longest, u.ntiles);
+        pl->coloc = static_cast<double>(longest + kTcItemCost) * tile_scale * kTileSec >= 5e-6;
+    }
     pl->pre_ctas = sms;
     if (pl->coloc) {
         int64_t dec_bytes = 0;
         for (const DecodeItem &it : ditems)
-            dec_bytes += static_cast<int64_t>(it.key_end - it.key_begin) * desc->num_kv_heads *
+            dec_bytes += static_cast<int64_t>(it.key_end - it.key_begin) * std::min(hpi, desc->num_kv_heads - it.kvh) *
                          (desc->kv_fp8 ? desc->head_dim_qk + desc->head_dim_v + 8
                                        : (desc->head_dim_qk + desc->head_dim_v) * 2);
         std::vector<int64_t> item_tiles;
         for (const TcUnit &u : tc_units) item_tiles.push_back(u.ntiles + kTcItemCost);
         std::sort(item_tiles.begin(), item_tiles.end(), [](int64_t a, int64_t b) { return a > b; });
-        const double tile_scale = (desc->head_dim_qk + desc->head_dim_v) / 256.0;  // relative to d = 128
         const int32_t k = o.decode_share_pct > 0
                               ? std::min(sms - 1, std::max(1, (sms * o.decode_share_pct + 50) / 100))
                               : choose_decode_sms(item_tiles, tile_scale, dec_bytes, sms);

@@ -11,7 +11,7 @@ namespace fnpu {
 
 // One decode split item: keys [key_begin, key_end) of sequence `seq` at the
 // sequence's single query position, for kv head `kvh` and its G query heads
-// (per-head kernel) or for every kv head (all-heads kernel, kvh = 0). Splits
+// (per-head kernel) or for the kv heads [kvh, kvh + 4) below Hkv (TMA kernel). Splits
 // of one group share `group` (their merge counter) and write partial results
 // to scratch rows part_base + split. The item also carries its sequence's
 // query token and block-table row and the ids of its first four blocks, so
@@ -167,6 +167,7 @@ bool decode_fp8_supported(int d_qk, int d_v, int hkv, int group, int block_size)
 int launch_decode_mma(const AttnParams &p, void *stream);
 int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas);
 bool decode_tma_supported(int d_qk, int d_v, int hkv, int group, int block_size);
+int decode_tma_heads_per_item();
 int launch_prefill_mma(const AttnParams &p, void *stream);
 int launch_mla(const AttnParams &p, void *stream);
 // tcgen05 latent attention: items are (token, d_v half, key range) of 128 heads

@@ -264,6 +264,22 @@ def test_decode_four_kv_heads_edges(bs, split):
     _compare(batch, out, lse)
 
 
+@pytest.mark.parametrize("dim,bs", [(64, 16), (128, 48)])
+@pytest.mark.parametrize("hkv", [1, 2, 3, 5, 8])
+def test_decode_kv_head_groups(hkv, dim, bs):
+    """Decode items cover groups of four kv heads: fewer than four, a ragged
+    last group and whole groups, alone and beside a prefill chunk, with split
+    lengths that are no multiple of a 16-key stage."""
+    sh = W.Shape(3 * hkv, hkv, dim, dim, bs, False)
+    ctx = [1, 15, 16, 17, 130, 700, 1501]
+    for n, (ql, c, ph) in enumerate([([], [], []), ([70], [270], [0])]):
+        rng = np.random.default_rng(100 * hkv + dim + n)
+        batch = W.build_batch(sh, ql + [1] * len(ctx), c + ctx, ph + [1] * len(ctx), rng, name="groups")
+        for split in (0, 100):
+            st = _step(batch, split=split)
+            _compare(batch, *st.results())
+
+
 @pytest.mark.parametrize("bs", [16, 64])
 @pytest.mark.parametrize("dim", [64, 128])
 def test_prefill_key_splits(bs, dim):
