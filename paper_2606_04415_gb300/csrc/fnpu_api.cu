@@ -500,6 +500,7 @@ namespace {
 // kernel drains, and its loaders wait for it before the first read.
 int launch_prefill(const fnpu_plan *pl, const AttnParams &p, void *stream, int ctas, void *started,
                    bool pdl = false) {
+    if (p.num_pitems == 0) return FNPU_OK;  // (nothing to stage either)
     if (!pl->desc.kv_fp8) return launch_prefill_tc(p, stream, ctas, started, false, pdl);
     const int rc = launch_fp8_stage(p.k_cache, p.v_cache, pl->d_jobs, pl->num_jobs, pl->d_tk, pl->d_tv, p.q, pl->d_tq,
                                     p.num_tokens * p.num_q_heads * p.head_dim_qk, stream);
