@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(kThreads, 3)
         tc::prefetch_tmap(&maps.k);
     }
     __syncthreads();
+    pdl_wait();  // the kernel before: the step's append, a writer of q, the last run's merge
 
     auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
         if (tc::mbar_try_wait(bar, parity)) return true;
@@ -450,7 +451,7 @@ bool decode_fp8_supported(int d_qk, int d_v, int hkv, int group, int block_size)
     return d_qk == kD && d_v == kD && hkv == kHkv && group <= 8 && block_size == kKeys;
 }
 
-int launch_decode_fp8(const AttnParams &p, void *stream, int max_ctas) {
+int launch_decode_fp8(const AttnParams &p, void *stream, int max_ctas, bool alone) {
     if (p.num_ditems == 0) return FNPU_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     Fp8Maps maps;
@@ -458,7 +459,7 @@ int launch_decode_fp8(const AttnParams &p, void *stream, int max_ctas) {
         return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled (fp8 decode)");
     FNPU_CUDA_TRY(cudaFuncSetAttribute(decode_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
     const int grid = p.num_ditems < max_ctas ? p.num_ditems : max_ctas;
-    FNPU_CUDA_TRY(launch_ex(decode_fp8_kernel, grid, kThreads, kSmemBytes, st, false, nullptr, p, maps));
+    FNPU_CUDA_TRY(launch_ex(decode_fp8_kernel, grid, kThreads, kSmemBytes, st, alone, nullptr, p, maps));
     return launch_split_merge(p, stream);
 }
 

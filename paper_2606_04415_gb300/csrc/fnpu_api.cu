@@ -711,6 +711,23 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
         int64_t sk = (dec_keys + target - 1) / std::max<int64_t>(target, 1);
         sk = (sk + 63) / 64 * 64;
         split = static_cast<int32_t>(std::min<int64_t>(std::max<int64_t>(sk, pl->use_dt ? 128 : 256), 4096));
+        if (pl->use_dt && split == 128) {
+            // A light batch: a CTA takes about 0.3 us per 16 keys, so halved
+            // items end sooner while they still start together (two per SM at
+            // most) and the merge still takes one pass (32 splits of a
+            // token): four decodes of 1400 keys 12.2 us a step against 13.5,
+            // 16 of 1000 13.7 against 14.1; past either line they lose: four
+            // of 4000 (63 splits) 16.5 against 14.9, 16 of 2000 (500 items)
+            // 20.4 against 16.5.
+            int64_t items = 0;
+            int32_t longest = 0;
+            for (int32_t s = 0; s < num_seqs; ++s)
+                if (decode_queue(s)) {
+                    items += static_cast<int64_t>((context_len[s] + 63) / 64) * hgroups;
+                    longest = std::max(longest, context_len[s]);
+                }
+            if (items <= 2LL * sms && longest <= 32 * 64) split = 64;
+        }
     }
 
     // latent attention: every query row (prefill or decode) is 64-head blocks
@@ -1252,7 +1269,7 @@ bool run_pointers_ok(const fnpu_plan *pl, const void *q, const void *k_cache, co
 
 // The decode kernel of a plan and its merge, on `stream`.
 int launch_decode(const fnpu_plan *pl, const AttnParams &p, void *stream, int ctas) {
-    return pl->desc.kv_fp8 ? launch_decode_fp8(p, stream, ctas) : launch_decode_tma(p, stream, ctas);
+    return pl->desc.kv_fp8 ? launch_decode_fp8(p, stream, ctas, false) : launch_decode_tma(p, stream, ctas, false);
 }
 
 // Both phases side by side: pre_ctas persistent prefill CTAs (one per SM, the
@@ -1327,7 +1344,7 @@ int run_step_fused(const fnpu_plan *pl, const AttnParams &p, const void *k_new, 
     }
     int rc = launch_kv_append_list(&pl->desc, k_new, v_new, slots, pl->d_dtok, pl->num_dtok, k_cache, v_cache, s);
     if (rc == FNPU_OK && pl->num_ditems > 0)
-        rc = pl->use_dt ? launch_decode_tma(p, stream, 3 * pl->num_sms) : launch_decode_mma(p, stream);
+        rc = pl->use_dt ? launch_decode_tma(p, stream, 3 * pl->num_sms, true) : launch_decode_mma(p, stream);
     if (rc != FNPU_OK) return rc;
     return launch_prefill(pl, p, stream, pl->num_sms, nullptr, false);
 }
@@ -1345,8 +1362,8 @@ int fnpu_mixed_attn_run(const fnpu_plan *pl, const void *q, const void *k_cache,
     const AttnParams p = run_params(pl, q, k_cache, v_cache, out, lse);
     if (pl->use_mla) return pl->use_mla_tc ? launch_mla_tc(p, stream) : launch_mla(p, stream);
     if (pl->coloc) return run_colocated(pl, p, stream);
-    int rc = pl->desc.kv_fp8 ? launch_decode_fp8(p, stream, 3 * pl->num_sms)
-             : pl->use_dt    ? launch_decode_tma(p, stream, 3 * pl->num_sms)
+    int rc = pl->desc.kv_fp8 ? launch_decode_fp8(p, stream, 3 * pl->num_sms, true)
+             : pl->use_dt    ? launch_decode_tma(p, stream, 3 * pl->num_sms, true)
                              : launch_decode_mma(p, stream);
     if (rc != FNPU_OK) return rc;
     if (pl->use_tc) return launch_prefill(pl, p, stream, pl->num_sms, nullptr, true);

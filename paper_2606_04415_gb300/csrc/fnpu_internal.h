@@ -153,7 +153,9 @@ int launch_mla_gather(const void *latent, const int64_t *slots, int32_t n, int64
 int launch_kv_append_fp8(const fnpu_attn_desc *d, const void *k_new, const void *v_new,
                          const int64_t *slots, int32_t num_tokens, void *k_cache, void *v_cache,
                          void *stream);
-int launch_decode_fp8(const AttnParams &p, void *stream, int max_ctas);
+// alone: the decode has the device to itself, as a programmatic dependent
+// launch of the kernel before it (else it follows events on its own stream)
+int launch_decode_fp8(const AttnParams &p, void *stream, int max_ctas, bool alone);
 int launch_prefill_fp8(const AttnParams &p, void *stream);
 // Staging of the FP8 cache for the tcgen05 prefill: job j dequantises source
 // block `src` (valid slots) into f16 block `dst` of k_f16 / v_f16 (plain
@@ -165,7 +167,7 @@ int launch_fp8_stage(const void *k_pool, const void *v_pool, const Fp8StageJob *
                      void *v_f16, const void *q_bf16, void *q_f16, int64_t q_values, void *stream);
 bool decode_fp8_supported(int d_qk, int d_v, int hkv, int group, int block_size);
 int launch_decode_mma(const AttnParams &p, void *stream);
-int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas);
+int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas, bool alone);
 bool decode_tma_supported(int d_qk, int d_v, int hkv, int group, int block_size);
 int decode_tma_heads_per_item();
 int launch_prefill_mma(const AttnParams &p, void *stream);

@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(256) kv_append_kernel(
     const int64_t *__restrict__ slots, int32_t num_tokens, int32_t k_chunks, int32_t v_chunks,
     uint4 *__restrict__ k_cache, uint4 *__restrict__ v_cache, int64_t num_slots) {
     pdl_trigger();  // a dependent launch after this one may start its set-up now
+    pdl_wait();     // earlier readers of the slots, writers of the rows
     const int32_t per_tok = k_chunks + v_chunks;
     const int64_t total = static_cast<int64_t>(num_tokens) * per_tok;
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total;
@@ -88,6 +89,8 @@ constexpr int kF8Block = kF8Codes + kF8Bs * kF8Hkv * 4;  // + fp32 scales [bs][H
 __global__ void __launch_bounds__(256) kv_append_fp8_kernel(
     const uint2 *__restrict__ k_new, const uint2 *__restrict__ v_new, const int64_t *__restrict__ slots,
     int32_t num_tokens, uint8_t *__restrict__ k_pool, uint8_t *__restrict__ v_pool, int64_t num_slots) {
+    pdl_trigger();  // as in kv_append_kernel
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nrows = static_cast<int64_t>(num_tokens) * 2 * kF8Hkv;
     const int64_t step = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -134,11 +137,11 @@ int launch_kv_append_fp8(const fnpu_attn_desc *d, const void *k_new, const void 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t want = (warps + 7) / 8;
     const int grid = static_cast<int>(want < 32LL * sms ? want : 32LL * sms);
-    kv_append_fp8_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint2 *>(k_new), static_cast<const uint2 *>(v_new), slots, num_tokens,
-        static_cast<uint8_t *>(k_cache), static_cast<uint8_t *>(v_cache),
-        static_cast<int64_t>(d->num_blocks) * kF8Bs);
-    return cudaGetLastError() == cudaSuccess ? FNPU_OK : FNPU_ECUDA;
+    FNPU_CUDA_TRY(launch_ex(kv_append_fp8_kernel, grid, 256, 0, static_cast<cudaStream_t>(stream), true, nullptr,
+                            static_cast<const uint2 *>(k_new), static_cast<const uint2 *>(v_new), slots, num_tokens,
+                            static_cast<uint8_t *>(k_cache), static_cast<uint8_t *>(v_cache),
+                            static_cast<int64_t>(d->num_blocks) * kF8Bs));
+    return FNPU_OK;
 }
 
 int launch_kv_append(const fnpu_attn_desc *d, const void *k_new, const void *v_new,
@@ -157,11 +160,11 @@ int launch_kv_append(const fnpu_attn_desc *d, const void *k_new, const void *v_n
     // latency-bound at step sizes, so every chunk should be in flight at once
     const int64_t want = (total + 255) / 256;
     const int grid = static_cast<int>(want < 32LL * sms ? want : 32LL * sms);
-    kv_append_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new), slots, num_tokens,
-        kc, vc, static_cast<uint4 *>(k_cache), static_cast<uint4 *>(v_cache),
-        static_cast<int64_t>(d->num_blocks) * d->block_size);
-    return cudaGetLastError() == cudaSuccess ? FNPU_OK : FNPU_ECUDA;
+    FNPU_CUDA_TRY(launch_ex(kv_append_kernel, grid, 256, 0, static_cast<cudaStream_t>(stream), true, nullptr,
+                            static_cast<const uint4 *>(k_new), static_cast<const uint4 *>(v_new), slots, num_tokens, kc,
+                            vc, static_cast<uint4 *>(k_cache), static_cast<uint4 *>(v_cache),
+                            static_cast<int64_t>(d->num_blocks) * d->block_size));
+    return FNPU_OK;
 }
 
 // The append of listed tokens only (the decode rows of a step whose prefill
