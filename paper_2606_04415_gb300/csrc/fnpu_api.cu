@@ -780,7 +780,7 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
                 for (int32_t sp = 0; sp < ns; ++sp)
                     for (int32_t h = 0; h < 2; ++h)  // the two d_v halves, next to each other
                         mitems.push_back(MlaItem{s, i, h, sp * per * kt, std::min(keys, (sp + 1) * per * kt), sp, ns,
-                                                 base, 0, 0, 0, 0});
+                                                 base, 0, qs + i, c, s});
             }
         } else if (pl->use_mla) {
             const int32_t nhb = desc->num_q_heads / mla_heads_per_item();
@@ -796,7 +796,7 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
                     }
                     for (int32_t sp = 0; sp < ns; ++sp)
                         mitems.push_back(MlaItem{s, i, hb, sp * sk, std::min(keys, (sp + 1) * sk), sp, ns, base, grp,
-                                                 0, 0, 0});
+                                                 qs + i, c, s});
                 }
             }
         } else if (decode_queue(s) && pl->use_dt) {
@@ -1360,7 +1360,7 @@ int fnpu_mixed_attn_run(const fnpu_plan *pl, const void *q, const void *k_cache,
     if (pl->num_tokens == 0) return FNPU_OK;
     if (!run_pointers_ok(pl, q, k_cache, v_cache, out, lse)) return FNPU_EINVAL;
     const AttnParams p = run_params(pl, q, k_cache, v_cache, out, lse);
-    if (pl->use_mla) return pl->use_mla_tc ? launch_mla_tc(p, stream) : launch_mla(p, stream);
+    if (pl->use_mla) return pl->use_mla_tc ? launch_mla_tc(p, stream, pl->num_sms) : launch_mla(p, stream);
     if (pl->coloc) return run_colocated(pl, p, stream);
     int rc = pl->desc.kv_fp8 ? launch_decode_fp8(p, stream, 3 * pl->num_sms, true)
              : pl->use_dt    ? launch_decode_tma(p, stream, 3 * pl->num_sms, true)

@@ -44,11 +44,13 @@ static_assert(sizeof(PrefillItem) == 64, "PrefillItem layout");
 // One latent-attention (MLA) work item: query heads [64 hb, 64 hb + 64) of
 // query row `row` of sequence `seq` (a prefill or a decode row alike) over
 // keys [key_begin, key_end); splits of one (token, head block) share `group`
-// and write partials to scratch rows part_base + split.
+// and write partials to scratch rows part_base + split. On the tcgen05 path hb
+// is the half of d_v (all 128 heads). The query token and the sequence's
+// context length and block-table row come along, so one load decodes an item.
 struct MlaItem {
     int32_t seq, row, hb, key_begin;
     int32_t key_end, split, num_splits, part_base;
-    int32_t group, pad0, pad1, pad2;
+    int32_t group, token, ctx_len, bt_row;
 };
 static_assert(sizeof(MlaItem) == 48, "MlaItem layout");
 
@@ -173,7 +175,7 @@ int decode_tma_heads_per_item();
 int launch_prefill_mma(const AttnParams &p, void *stream);
 int launch_mla(const AttnParams &p, void *stream);
 // tcgen05 latent attention: items are (token, d_v half, key range) of 128 heads
-int launch_mla_tc(const AttnParams &p, void *stream);
+int launch_mla_tc(const AttnParams &p, void *stream, int max_ctas);
 bool mla_tc_supported(int d_qk, int d_v, int hq, int hkv, int block_size);
 int mla_tc_keys_per_tile();
 // log-sum-exp merge of the split tokens listed in p.mgroups (partials [part, Hq, dv])

@@ -347,6 +347,22 @@ def test_mla_small_mixed_batch_all_rows(bs, flags):
     assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
 
 
+@pytest.mark.parametrize("bs", [16, 64])
+@pytest.mark.parametrize("tokens", [1, 75, 77, 230])
+def test_mla_items_around_the_grid(tokens, bs):
+    """The persistent latent kernel with fewer, about as many and several
+    times as many items as CTAs, of one to four key tiles, off tile edges."""
+    sh = W.Shape(128, 1, 576, 512, bs, True)
+    rng = np.random.default_rng(tokens + bs)
+    batch = W.build_batch(sh, [tokens, 1, 1], [tokens, 64, 65], [0, 1, 1], rng, name="mla_grid")
+    st = _step(batch)
+    out, lse = st.results()
+    _compare(batch, out, lse)
+    st.run()
+    out2, lse2 = st.results()
+    assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
+
+
 def test_mla_coloc_full_size_sampled_rows():
     """The DeepSeek-R1-shaped co-located step at full size (1024-token
     prefill + 256 decodes up to 16K keys); the oracle recomputes a sample of
