@@ -313,7 +313,9 @@ int fnpu_plan_decode_share(const fnpu_plan *plan, int32_t *share_pct);
  *   block_table   device int32 [num_seqs, block_table_stride], stride >=
  *                 ceil(max_context_len / block_size)
  *   max_context_len  host bound on context_len; it sizes the grid
- *   split_keys    keys per split, a multiple of 64; 0 selects 512
+ *   split_keys    keys per split, a multiple of 64; 0 leaves it to the library
+ *                 (256 or 128 for light batches where the scratch allows, else
+ *                 512; requests are accepted or refused as for 512)
  *   q             device bf16 [num_seqs, Hq, d]; out bf16 [num_seqs, Hq, d];
  *                 lse fp32 [num_seqs, Hq]; k_cache / v_cache as above
  * Supports split K/V caches with d_qk = d_v in {64, 128} and Hq/Hkv <= 8.
@@ -333,8 +335,8 @@ int fnpu_plan_decode_share(const fnpu_plan *plan, int32_t *share_pct);
  * The first call on a device looks up the scratch array's device address
  * (cudaGetSymbolAddress) while that device is current; make that first call
  * before any stream capture. All calls share the one array, which keeps the
- * last call's contents; each call clears its merge counters itself with
- * cudaMemsetAsync on `stream`. Calls that overlap on the GPU (on different
+ * last call's contents; a call that merges by counters (block sizes that are
+ * no multiple of 16) clears them itself with cudaMemsetAsync on `stream`. Calls that overlap on the GPU (on different
  * streams, or with no ordering between them) race on the array and must not
  * be issued.
  */

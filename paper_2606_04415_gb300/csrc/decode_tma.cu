@@ -47,6 +47,12 @@
 //     capped the splits per sequence, and with few splits the items were too
 //     coarse to share the bandwidth evenly among the CTAs.
 // Every mbarrier wait is bounded and raises the plan's error flag on timeout.
+//
+// The allocation-free decode (fnpu_decode_attn_noalloc) runs the same kernel
+// without a plan (kNoPlan): item i is split i / (sequences x head groups) of
+// a sequence and head group, CTA b takes items b, b + grid, ... that its
+// sequence's context reaches, and lengths and block ids, which are device
+// data, are checked as they are read.
 #include <math.h>
 
 #include "common.cuh"
@@ -117,7 +123,7 @@ __device__ __forceinline__ int load_blk_lane(const AttnParams &p, const DtGeo &g
 
 // kRagged: the kv heads are no multiple of four, so that a warp of the last
 // group may have none (the checks cost a small step 7% where they are not needed)
-template <int D, bool kRagged, int kStages>
+template <int D, bool kRagged, int kStages, bool kNoPlan>
 __global__ void __launch_bounds__(kThreads, 3)
     decode_tma_kernel(const AttnParams p, const __grid_constant__ DtMaps maps) {
     using Cfg = DtCfg<D, kStages>;
@@ -133,16 +139,60 @@ __global__ void __launch_bounds__(kThreads, 3)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n_items = p.num_ditems;
     pdl_trigger();  // the merge grid may be placed once these CTAs are; it waits for them to finish
+    // (the library-wide flag of a run without a plan has its own bit for timeouts)
+    constexpr int kErrTimeout = kNoPlan ? 4 : 1, kErrAlign = kNoPlan ? 4 : 2;
     if ((s_base & 1023u) != 0) {  // the swizzled tiles need 1024-byte alignment
-        if (tid == 0) atomicOr(p.err, 2);
+        pdl_wait();
+        if (tid == 0) atomicOr(p.err, kErrAlign);
         return;
     }
+    // without a plan: item i from the device's lengths; false where the
+    // sequence's context does not reach it (or is out of range: flagged once)
+    auto noplan_item = [&](int i, DecodeItem &it) -> bool {
+        const int groups = (p.num_kv_heads + kHkv - 1) / kHkv, per = p.na_num_seqs * groups;
+        const int split = i / per, r = i - split * per, seq = r / groups, hg = r - seq * groups;
+        const int ctx = p.na_ctx[seq];
+        if (ctx < 1 || ctx > p.na_max_ctx) {
+            if (split == 0 && hg == 0) atomicOr(p.err, 2);
+            return false;
+        }
+        const int kb = split * p.na_split;
+        if (kb >= ctx) return false;
+        it.seq = it.q_start = it.bt_row = seq;
+        it.kvh = hg * kHkv;
+        it.key_begin = kb;
+        it.key_end = kb + p.na_split < ctx ? kb + p.na_split : ctx;
+        it.split = split;
+        it.num_splits = (ctx + p.na_split - 1) / p.na_split;
+        it.part_base = seq * p.na_max_splits;
+        it.group = 0;
+        const int b0 = kb / p.block_size, b1 = (it.key_end - 1) / p.block_size;
+        for (int j = 0; j < 4; ++j)
+            it.blk[j] = b0 + j <= b1 ? p.block_table[static_cast<int64_t>(seq) * p.bt_stride + b0 + j] : 0;
+        return true;
+    };
+    auto noplan_next = [&](int i) -> int {  // the first item from i on, in steps of the grid, that there is
+        DecodeItem it;
+        while (i < n_items && !noplan_item(i, it)) i += static_cast<int>(gridDim.x);
+        return i < n_items ? i : n_items;
+    };
+    auto item_at = [&](int i) -> DecodeItem {
+        if constexpr (kNoPlan) {
+            DecodeItem it{};
+            noplan_item(i, it);
+            return it;
+        } else {
+            return p.ditems[i];
+        }
+    };
+    if (kNoPlan) pdl_wait();  // lengths and block ids may come from the kernel before
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             tc::mbar_init(FULL(s), 1);
             tc::mbar_init(EMPTY(s), kWarps);
         }
-        ring[0] = blockIdx.x;  // the first item without the queue (grid <= items); the queue serves the rest
+        // the first item without the queue (grid <= items); the queue serves the rest
+        ring[0] = kNoPlan ? noplan_next(blockIdx.x) : static_cast<int>(blockIdx.x);
         *abort_flag = 0;
         tc::fence_mbar_init();
     }
@@ -158,7 +208,7 @@ __global__ void __launch_bounds__(kThreads, 3)
         if (*abort_flag) return false;
         if (tc::mbar_wait(bar, parity)) return true;
         *abort_flag = 1;
-        atomicOr(p.err, 1);
+        atomicOr(p.err, kErrTimeout);
         return false;
     };
     auto geo_of = [&](const DecodeItem &it) {
@@ -203,6 +253,11 @@ __global__ void __launch_bounds__(kThreads, 3)
             blk = __shfl_sync(0xffffffffu, blk_lane, rel & 31);
             if (rel >= 32) blk = __ldg(p.block_table + static_cast<int64_t>(g.bt_row) * p.bt_stride + key0 / bs);
         }
+        if (kNoPlan && static_cast<uint32_t>(blk) >= static_cast<uint32_t>(p.num_blocks)) {
+            // never loaded: the copy of a block past the last fills zeros
+            if (lane == 0) atomicOr(p.err, 2);
+            blk = p.num_blocks;
+        }
         const uint32_t sK = s_base + st * Cfg::kStageBytes, sV = sK + Cfg::kTileBytes;
         tc::mbar_arrive_expect_tx_warp(FULL(st), stage_bytes);
 #pragma unroll
@@ -227,12 +282,12 @@ __global__ void __launch_bounds__(kThreads, 3)
         bool ok = true;
         int idx = ring[0];
         DecodeItem it{};
-        if (idx < n_items) it = p.ditems[idx];
+        if (idx < n_items) it = item_at(idx);
         DtGeo cur = geo_of(it);
         int blk_lane = idx < n_items ? load_blk_lane(p, cur, lane) : 0;
         for (int k = 0; ok && idx < n_items; ++k) {
             int a = 0;
-            if (lane == 0) a = static_cast<int>(gridDim.x) + atomicAdd(sched, 1);  // the next item
+            if (!kNoPlan && lane == 0) a = static_cast<int>(gridDim.x) + atomicAdd(sched, 1);  // the next item
             const int ntiles = (cur.ke - cur.kb + kKeys - 1) / kKeys;
             const int spub = ntiles > 2 ? 2 : ntiles - 1;
             const int s1 = spub + 1 < ntiles ? spub + 1 : spub;
@@ -242,10 +297,11 @@ __global__ void __launch_bounds__(kThreads, 3)
             int blk_lane_n = 0;
             for (int i = 0; i < ntiles; ++i, ++gs) {
                 if (i == spub) {
+                    if (kNoPlan && lane == 0) a = noplan_next(idx + static_cast<int>(gridDim.x));
                     idx_n = __shfl_sync(0xffffffffu, a, 0);
                     if (lane == 0) *reinterpret_cast<volatile int *>(ring + ((k + 1) & 3)) = idx_n;
                     __syncwarp();  // before the arrival of this stage, which releases it
-                    if (idx_n < n_items) nit = p.ditems[idx_n];
+                    if (idx_n < n_items) nit = item_at(idx_n);
                 }
                 if (!issue(cur, i, blk_lane, gs)) { ok = false; break; }
                 if (idx_n < n_items && i == s1) {
@@ -262,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, 3)
         int idx = ring[0];
         DtGeo cur;
         {
-            cur = geo_of(p.ditems[idx]);
+            cur = geo_of(item_at(idx));
         }
         uint32_t qb[D / 16][2];
         if (has_head(cur)) load_q<D>(p, cur.t, cur.head0 + wh, g8, c, qb);
@@ -289,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 3)
                 if (i == spub) {  // the producer published it before issuing this stage
                     idx_n = *reinterpret_cast<volatile int *>(ring + ((k + 1) & 3));
                     has_next = idx_n < n_items;
-                    if (has_next) nit = p.ditems[idx_n];
+                    if (has_next) nit = item_at(idx_n);
                 }
                 const uint32_t sK = s_base + st * Cfg::kStageBytes, sV = sK + Cfg::kTileBytes;
                 const int nv = nkeys - i * kKeys;  // valid keys in this stage (>= 1)
@@ -412,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     }
 
     __syncthreads();
-    if (tid == 0) {  // the last CTA out resets the work queue for the next run
+    if (!kNoPlan && tid == 0) {  // the last CTA out resets the work queue for the next run
         __threadfence();
         if (atomicAdd(sched + 1, 1) == static_cast<int>(gridDim.x) - 1) {
             sched[0] = 0;
@@ -432,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 3)
 // flight, so a token of up to 32 splits costs a few memory round trips.
 constexpr int kMergeWarps = 4;
 
-template <int D>
+template <int D, bool kNoPlan>
 __global__ void __launch_bounds__(32 * kMergeWarps) split_merge_kernel(const AttnParams p) {
     constexpr int kV = D / 4;                 // float4 per row
     constexpr int kC = (kV + 31) / 32;        // float4 columns per lane
@@ -442,7 +498,16 @@ __global__ void __launch_bounds__(32 * kMergeWarps) split_merge_kernel(const Att
     pdl_trigger();  // (the next step's append may be placed; it waits for this grid to finish)
     pdl_wait();     // the partial results of the grid before
     if (wg >= p.num_mgroups * Hq) return;
-    const MergeGroup mg = p.mgroups[wg / Hq];
+    MergeGroup mg;
+    if constexpr (kNoPlan) {
+        mg.token = wg / Hq;
+        const int ctx = p.na_ctx[mg.token];
+        if (ctx <= p.na_split || ctx > p.na_max_ctx) return;  // one split: already written; out of range: skipped
+        mg.num_splits = (ctx + p.na_split - 1) / p.na_split;
+        mg.part_base = mg.token * p.na_max_splits;
+    } else {
+        mg = p.mgroups[wg / Hq];
+    }
     const int h = wg % Hq;
     const int ns = mg.num_splits, base = mg.part_base;
     const float4 *po = reinterpret_cast<const float4 *>(p.part_o);
@@ -522,10 +587,10 @@ bool encode_slot_major_map(CUtensorMap *m, const void *base, int d, int hkv, int
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, bool kRagged, int kStages>
+template <int D, bool kRagged, int kStages, bool kNoPlan>
 int launch_dt(const AttnParams &p, cudaStream_t st, int grid, bool after_prev) {
     using Cfg = DtCfg<D, kStages>;
-    auto kernel = decode_tma_kernel<D, kRagged, kStages>;
+    auto kernel = decode_tma_kernel<D, kRagged, kStages, kNoPlan>;
     DtMaps maps;
     if (!encode_slot_major_map(&maps.k, p.k_cache, D, p.num_kv_heads, p.block_size, p.num_blocks) ||
         !encode_slot_major_map(&maps.v, p.v_cache, D, p.num_kv_heads, p.block_size, p.num_blocks))
@@ -539,13 +604,44 @@ int launch_dt(const AttnParams &p, cudaStream_t st, int grid, bool after_prev) {
 
 // The ring depth: an SM's shared memory holds six 32 KB stages (d = 128), and
 // all of them should be in flight whatever the number of CTAs on it.
-template <int D, bool kRagged>
+template <int D, bool kRagged, bool kNoPlan>
 int launch_dt(const AttnParams &p, cudaStream_t st, int max_ctas, bool alone) {
     const int grid = p.num_ditems < max_ctas ? p.num_ditems : max_ctas;
     const int sms = max_ctas / 3;
-    if (alone && grid <= sms) return launch_dt<D, kRagged, 6>(p, st, grid, alone);
-    if (alone && grid <= 2 * sms) return launch_dt<D, kRagged, 3>(p, st, grid, alone);
-    return launch_dt<D, kRagged, 2>(p, st, grid, alone);
+    if (alone && grid <= sms) return launch_dt<D, kRagged, 6, kNoPlan>(p, st, grid, alone);
+    if (alone && grid <= 2 * sms) return launch_dt<D, kRagged, 3, kNoPlan>(p, st, grid, alone);
+    return launch_dt<D, kRagged, 2, kNoPlan>(p, st, grid, alone);
+}
+
+template <bool kNoPlan>
+int launch_dt_shape(const AttnParams &p, cudaStream_t st, int max_ctas, bool alone) {
+    const bool ragged = p.num_kv_heads % kHkv != 0;
+    switch (p.head_dim_qk) {
+        case 64:
+            return ragged ? launch_dt<64, true, kNoPlan>(p, st, max_ctas, alone)
+                          : launch_dt<64, false, kNoPlan>(p, st, max_ctas, alone);
+        case 128:
+            return ragged ? launch_dt<128, true, kNoPlan>(p, st, max_ctas, alone)
+                          : launch_dt<128, false, kNoPlan>(p, st, max_ctas, alone);
+        default: return FNPU_EUNSUPPORTED;
+    }
+}
+
+template <bool kNoPlan>
+int launch_merge(const AttnParams &p, cudaStream_t st) {
+    const int blocks = (p.num_mgroups * p.num_q_heads + kMergeWarps - 1) / kMergeWarps;
+    void (*kernel)(AttnParams) = nullptr;
+    switch (p.head_dim_v) {
+        case 64: kernel = split_merge_kernel<64, kNoPlan>; break;
+        case 128: kernel = split_merge_kernel<128, kNoPlan>; break;
+        case 512: kernel = kNoPlan ? nullptr : split_merge_kernel<512, false>; break;
+        default: break;
+    }
+    if (!kernel) return FNPU_EUNSUPPORTED;
+    // a dependent launch: its CTAs take the SMs that the CTAs of the grid
+    // before leave and wait there for that grid's writes
+    FNPU_CUDA_TRY(launch_ex(kernel, blocks, 32 * kMergeWarps, 0, st, true, nullptr, p));
+    return FNPU_OK;
 }
 
 }  // namespace
@@ -559,38 +655,21 @@ int decode_tma_heads_per_item() { return kHkv; }
 
 int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas, bool alone) {
     if (p.num_ditems == 0) return FNPU_OK;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int rc = FNPU_EUNSUPPORTED;
-    switch (p.head_dim_qk) {
-        case 64:
-            rc = p.num_kv_heads % kHkv ? launch_dt<64, true>(p, st, max_ctas, alone)
-                                       : launch_dt<64, false>(p, st, max_ctas, alone);
-            break;
-        case 128:
-            rc = p.num_kv_heads % kHkv ? launch_dt<128, true>(p, st, max_ctas, alone)
-                                       : launch_dt<128, false>(p, st, max_ctas, alone);
-            break;
-        default: break;
-    }
+    const int rc = launch_dt_shape<false>(p, static_cast<cudaStream_t>(stream), max_ctas, alone);
     if (rc != FNPU_OK) return rc;
     return launch_split_merge(p, stream);
 }
 
+int launch_decode_tma_noplan(const AttnParams &p, void *stream, int max_ctas) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const int rc = launch_dt_shape<true>(p, st, max_ctas, true);
+    if (rc != FNPU_OK || p.na_max_splits == 1) return rc;
+    return launch_merge<true>(p, st);
+}
+
 int launch_split_merge(const AttnParams &p, void *stream) {
     if (p.num_mgroups == 0) return FNPU_OK;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int blocks = (p.num_mgroups * p.num_q_heads + kMergeWarps - 1) / kMergeWarps;
-    void (*kernel)(AttnParams) = nullptr;
-    switch (p.head_dim_v) {
-        case 64: kernel = split_merge_kernel<64>; break;
-        case 128: kernel = split_merge_kernel<128>; break;
-        case 512: kernel = split_merge_kernel<512>; break;
-        default: return FNPU_EUNSUPPORTED;
-    }
-    // a dependent launch: its CTAs take the SMs that the CTAs of the grid
-    // before leave and wait there for that grid's writes
-    FNPU_CUDA_TRY(launch_ex(kernel, blocks, 32 * kMergeWarps, 0, st, true, nullptr, p));
-    return FNPU_OK;
+    return launch_merge<false>(p, static_cast<cudaStream_t>(stream));
 }
 
 }  // namespace fnpu

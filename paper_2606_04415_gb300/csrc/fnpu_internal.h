@@ -118,6 +118,12 @@ struct AttnParams {
     int *fa_range_err;      // the library-wide error flag (bit 0: a slot past the pool)
     int32_t fa_num_tokens, fa_k_chunks, fa_v_chunks;
     int64_t fa_num_slots;
+    // decode without a plan (one query row per sequence): context lengths on
+    // the device, the host's bound on them, keys per split and the splits that
+    // bound allows; err is the library-wide flag (bit 1: out of range, bit 2:
+    // a wait that gave up)
+    const int32_t *na_ctx;
+    int32_t na_num_seqs, na_max_ctx, na_split, na_max_splits;
 };
 
 // cuTensorMapEncodeTiled, looked up once through the runtime's driver entry
@@ -172,6 +178,9 @@ int launch_decode_mma(const AttnParams &p, void *stream);
 int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas, bool alone);
 bool decode_tma_supported(int d_qk, int d_v, int hkv, int group, int block_size);
 int decode_tma_heads_per_item();
+// without a plan: p.na_*, num_ditems = sequences x head groups x na_max_splits,
+// num_mgroups = sequences, partial rows sequence x na_max_splits + split
+int launch_decode_tma_noplan(const AttnParams &p, void *stream, int max_ctas);
 int launch_prefill_mma(const AttnParams &p, void *stream);
 int launch_mla(const AttnParams &p, void *stream);
 // tcgen05 latent attention: items are (token, d_v half, key range) of 128 heads

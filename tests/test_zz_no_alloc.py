@@ -164,3 +164,31 @@ def test_noalloc_skips_and_flags_out_of_range_context_and_block():
     for s in (0, 3):
         assert np.abs(o[s] - ref_o[s]).max() <= O_TOL
         assert np.abs(l[s] - ref_l[s]).max() <= LSE_TOL
+
+
+@pytest.mark.parametrize("bs", [16, 48, 24])
+@pytest.mark.parametrize("heads", [(8, 8), (9, 3), (35, 5), (28, 4)])
+@pytest.mark.parametrize("split_keys", [0, 64])
+def test_noalloc_head_groups_block_sizes_and_split_lengths(heads, bs, split_keys):
+    """One, several and a ragged last group of kv heads; block sizes on the
+    TMA-fed path and (24) off it; contexts at split and stage edges, one of
+    them the bound itself, with open and given split lengths."""
+    _need_gpu()
+    import paper_2606_04415_gb300 as fnpu
+    from paper_2606_04415_gb300.step import DeviceStep
+    hq, hkv = heads
+    sh = W.Shape(hq, hkv, 128, 128, bs, False)
+    ctx = [1, 16, 17, 63, 64, 65, 128, 129, 512, 513, 1300]
+    rng = np.random.default_rng(10 * hkv + bs)
+    batch = W.build_batch(sh, [1] * len(ctx), ctx, [1] * len(ctx), rng, name="noalloc_groups")
+    st = DeviceStep(batch)
+    st.append()
+    out = torch.full_like(st.out, float("nan"))
+    lse = torch.full_like(st.lse, float("nan"))
+    fnpu.decode_attn_noalloc(st.desc, torch.from_numpy(batch.context_len).cuda(), torch.from_numpy(batch.block_table).cuda(),
+                             1300, st.q, st.k_cache, st.v_cache, out, lse, split_keys=split_keys)
+    torch.cuda.synchronize()
+    assert fnpu.check() == fnpu.FNPU_OK
+    ref_o, ref_l = _oracle_after_append(batch)
+    assert np.abs(out.float().cpu().numpy() - ref_o).max() <= O_TOL
+    assert np.abs(lse.cpu().numpy() - ref_l).max() <= LSE_TOL
