@@ -35,8 +35,9 @@
 //   warps 0-3  softmax, one row each (TMEM lane = head), with a lazy O rescale
 //              (only when the row maximum grows by more than 2^8), while no
 //              product is writing O: when S(j) is complete so is P V(j - 1);
-//   warp 4     scheduler and TMA producer: the next item's first tiles load
-//              while the current one ends;
+//   warp 4     scheduler and TMA producer (each lane issues one box of a part,
+//              so that a tile of four 16-slot blocks is no slower): the next
+//              item's first tiles load while the current one ends;
 //   warp 5     MMA issuer;
 //   warps 6-9  the next item's tensor-memory part of Q (held in registers
 //              until the last S of the current item is done) and the epilogue
@@ -209,24 +210,26 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
                 const int st = gt % kStages;
                 if (gt >= kStages && !wait(NEMPTY(st), ((gt / kStages) - 1) & 1)) { ok = false; break; }
                 tc::mbar_arrive_expect_tx_warp(NFULL(st), static_cast<uint32_t>(nvalid * bs * 128 * kNChunks));
-#pragma unroll 1
-                for (int b = 0; b < nvalid; ++b) {  // the chunks that only S reads
+                __syncwarp();
+                {  // the chunks that only S reads, one copy (block, chunk) a lane
+                    const int b = lane / kNChunks, c = lane % kNChunks;
                     const int blk = __shfl_sync(0xffffffffu, blk_cur, b);
-#pragma unroll 1
-                    for (int c = 0; c < kNChunks; ++c)
-                        tc::tma_load_3d_warp(s_base + kOffN + st * kNBytes + c * kChunkBytes + b * bs * 128, &maps.kv,
-                                             NFULL(st), 64 * (c < 4 ? 4 * (1 - half) + c : 8), 0, blk);
+                    if (b < nvalid)
+                        tc::tma_load_3d(s_base + kOffN + st * kNBytes + c * kChunkBytes + b * bs * 128, &maps.kv, NFULL(st),
+                                        64 * (c < 4 ? 4 * (1 - half) + c : 8), 0, blk);
+                    __syncwarp();
                 }
                 ++gt;
                 if (gv >= kStages && !wait(VEMPTY(st), ((gv / kStages) - 1) & 1)) { ok = false; break; }
                 tc::mbar_arrive_expect_tx_warp(VFULL(st), static_cast<uint32_t>(nvalid * bs * 128 * kVChunks));
-#pragma unroll 1
-                for (int b = 0; b < nvalid; ++b) {  // the chunks of this half's V
+                __syncwarp();
+                {  // the chunks of this half's V
+                    const int b = lane / kVChunks, c = lane % kVChunks;
                     const int blk = __shfl_sync(0xffffffffu, blk_cur, b);
-#pragma unroll 1
-                    for (int c = 0; c < kVChunks; ++c)
-                        tc::tma_load_3d_warp(s_base + kOffV + st * kVBytes + c * kChunkBytes + b * bs * 128, &maps.kv,
-                                             VFULL(st), 64 * (4 * half + c), 0, blk);
+                    if (b < nvalid)
+                        tc::tma_load_3d(s_base + kOffV + st * kVBytes + c * kChunkBytes + b * bs * 128, &maps.kv, VFULL(st),
+                                        64 * (4 * half + c), 0, blk);
+                    __syncwarp();
                 }
                 ++gv;
                 if (j == 0) {  // the other half's Q columns, once the previous item's last S is done
