@@ -220,11 +220,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int w = 0; w < 2; ++w) {
             tc::mbar_init(SFULL(w), 1);
-            tc::mbar_init(PFULL(w), kRows);
+            tc::mbar_init(PFULL(w), 4);  // one arrival a softmax warp
             tc::mbar_init(ODONE(w), 1);
-            tc::mbar_init(OFREE(w), kRows);
+            tc::mbar_init(OFREE(w), 4);
             tc::mbar_init(ITEMFULL(w), 1);
-            tc::mbar_init(ITEMEMPTY(w), 2 + 2 * kRows);  // MMA issuer, V producer, 256 softmax rows
+            tc::mbar_init(ITEMEMPTY(w), 2 + 8);  // MMA issuer, V producer, eight softmax warps
         }
         tc::mbar_init(QFULL, 1);
         tc::mbar_init(QEMPTY, 1);
@@ -323,36 +323,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 nvalid = nvalid < 0 ? 0 : (nvalid > per_tile ? per_tile : nvalid);
                 nvalid = __shfl_sync(0xffffffffu, nvalid, 0);
                 const uint32_t bar = is_k ? KFULL(st) : VFULL(st);
-                if constexpr (DQ == DV) {
-                    const uint32_t dst = s_base + (is_k ? 0 : Cfg::kVOff) + st * Cfg::kKTileBytes;
-                    tc::mbar_arrive_expect_tx_warp(bar, static_cast<uint32_t>(nvalid) * bs * DQ * 2);
-                    for (int b = 0; b < per_tile; ++b) {
-                        const int blk = __shfl_sync(0xffffffffu, blk_cur, b);
-                        if (b < nvalid) {
-#pragma unroll
-                            for (int h = 0; h < DQ / 64; ++h)
-                                tc::tma_load_4d_warp(dst + h * Cfg::kHalf + b * bs * 128, map, bar, h * 64, ukvh, 0, blk);
-                        }
-                    }
-                } else {
-                    const uint32_t dst = s_base + (is_k ? st * Cfg::kKTileBytes : Cfg::kVOff + st * Cfg::kVTileBytes);
-                    const int dcols = is_k ? DQ : DV;
-                    tc::mbar_arrive_expect_tx_warp(bar, static_cast<uint32_t>(nvalid) * bs * dcols * 2);
-                    for (int b = 0; b < per_tile; ++b) {
-                        const int blk = __shfl_sync(0xffffffffu, blk_cur, b);
-                        if (b < nvalid) {
-                            if (is_k) {
-#pragma unroll
-                                for (int h = 0; h < DQ / 64; ++h)
-                                    tc::tma_load_4d_warp(dst + h * Cfg::kHalf + b * bs * 128, map, bar, h * 64, ukvh, 0, blk);
-                            } else {
-#pragma unroll
-                                for (int h = 0; h < DV / 64; ++h)
-                                    tc::tma_load_4d_warp(dst + h * Cfg::kHalf + b * bs * 128, map, bar, h * 64, ukvh, 0, blk);
-                            }
-                        }
-                    }
-                }
+                // one box (block, 64-column chunk) a lane: at most 8 x 3
+                const int nch = is_k ? DQ / 64 : DV / 64, lb = lane / nch, lh = lane % nch;
+                const int blk = __shfl_sync(0xffffffffu, blk_cur, lb & 31);
+                const uint32_t dst = s_base + (is_k ? st * Cfg::kKTileBytes : Cfg::kVOff + st * Cfg::kVTileBytes);
+                tc::mbar_arrive_expect_tx_warp(bar, static_cast<uint32_t>(nvalid) * bs * nch * 128);
+                __syncwarp();
+                if (lb < nvalid) tc::tma_load_4d(dst + lh * Cfg::kHalf + lb * bs * 128, map, bar, lh * 64, ukvh, 0, blk);
+                __syncwarp();
                 if (!is_k && i == it.ntiles - 1 && it.tail_fix) {
                     // zero V rows of keys >= ctx (stale slots, unloaded blocks)
                     if (!wait(VFULL(st), (g / nst) & 1)) { ok = false; break; }
@@ -375,36 +353,42 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == 10) {
         // -------------------------------------------------------- MMA issuer
-        // The loop runs with warp-uniform values (passed through __shfl_sync
-        // so the compiler keeps them in uniform registers); each tcgen05
-        // instruction is issued by one elected lane.
+        // One elected lane issues the products of a burst inside one branch:
+        // electing a lane for each took 29 instructions a product, and the
+        // issuer's 15 KB a step and the softmax evicted each other from the
+        // instruction cache. With that, one place in the code per product and
+        // one box per producer lane, the step of 2048 tokens on a prefix of
+        // 7000 beside 128 decodes takes 197 us (205 before), four 512-token
+        // chunks 34.5 (39.1).
         constexpr uint32_t idS = F16 ? tc::idesc_f16(kRows, kKeys, false) : tc::idesc_bf16(kRows, kKeys, false);
         constexpr uint32_t idO = F16 ? tc::idesc_f16(kRows, DV, true) : tc::idesc_bf16(kRows, DV, true);
         const uint32_t utmem = __shfl_sync(0xffffffffu, tmem, 0);
         const uint32_t us_base = __shfl_sync(0xffffffffu, s_base, 0);
         int gk = 0, gv = 0, t = 0, nfix = 0;
         bool ok = true, issued = false;
-        auto issue_s = [&](int w, int st_in) {
-            const int st = __shfl_sync(0xffffffffu, st_in, 0);
-            const uint64_t kd = tc::sdesc_sw128(us_base + st * Cfg::kKTileBytes, 16, 1024);
-            const uint64_t qd = tc::sdesc_sw128(us_base + Cfg::kQOff + w * Cfg::kQBytes, 16, 1024);
-            const uint32_t dS = utmem + col_s(w);
+        auto issue_s = [&](int w, int st) {
+            if (tc::elect_one()) {
+                const uint64_t kd = tc::sdesc_sw128(us_base + st * Cfg::kKTileBytes, 16, 1024);
+                const uint64_t qd = tc::sdesc_sw128(us_base + Cfg::kQOff + w * Cfg::kQBytes, 16, 1024);
+                const uint32_t dS = utmem + col_s(w);
 #pragma unroll
-            for (int kk = 0; kk < DQ / 16; ++kk)
-                tc::mma_ss_warp(dS, qd + ((kk / 4) * Cfg::kQHalf + (kk % 4) * 32) / 16,
-                                kd + ((kk / 4) * Cfg::kHalf + (kk % 4) * 32) / 16, idS, kk > 0);
-            tc::commit_warp(SFULL(w));
+                for (int kk = 0; kk < DQ / 16; ++kk)
+                    tc::mma_ss(dS, qd + ((kk / 4) * Cfg::kQHalf + (kk % 4) * 32) / 16,
+                               kd + ((kk / 4) * Cfg::kHalf + (kk % 4) * 32) / 16, idS, kk > 0);
+                tc::commit(SFULL(w));
+            }
+            __syncwarp();
             issued = true;
         };
-        auto issue_pv = [&](int w, int st_in, uint32_t acc_in) {
-            const int st = __shfl_sync(0xffffffffu, st_in, 0);
-            const uint32_t acc = __shfl_sync(0xffffffffu, acc_in, 0);
-            const uint64_t vd =
-                tc::sdesc_sw128(us_base + Cfg::kVOff + st * Cfg::kVTileBytes, Cfg::kHalf, 1024);
-            const uint32_t dO = utmem + col_o(w), aP = utmem + col_s(w);
-            tc::mma_ts_warp(dO, aP, vd, idO, acc);
+        auto issue_pv = [&](int w, int st, uint32_t acc) {
+            if (tc::elect_one()) {
+                const uint64_t vd = tc::sdesc_sw128(us_base + Cfg::kVOff + st * Cfg::kVTileBytes, Cfg::kHalf, 1024);
+                const uint32_t dO = utmem + col_o(w), aP = utmem + col_s(w);
+                tc::mma_ts(dO, aP, vd, idO, acc);
 #pragma unroll
-            for (int kk = 1; kk < kKeys / 16; ++kk) tc::mma_ts_warp(dO, aP + kk * 8, vd + (kk * 2048) / 16, idO, 1u);
+                for (int kk = 1; kk < kKeys / 16; ++kk) tc::mma_ts(dO, aP + kk * 8, vd + (kk * 2048) / 16, idO, 1u);
+            }
+            __syncwarp();
             issued = true;
         };
         for (int k = 0; ok; ++k) {
@@ -415,56 +399,54 @@ __global__ void __launch_bounds__(kThreads, 1)
             const ItemGeom it = item_geom(p, idx);
             const int n = __shfl_sync(0xffffffffu, it.ntiles, 0);
             const bool tail = __shfl_sync(0xffffffffu, it.tail_fix ? 1 : 0, 0) != 0;
-            // S_0(0), S_1(0)
+            // PV_0(u - 1), S_0(u), PV_1(u - 1), S_1(u) for u = 0 .. n: each product
+            // has one place in the code, so that the issuer takes little of the
+            // instruction cache that it shares with the softmax
             if (!wait(QFULL, k & 1)) { ok = false; break; }
-            if (!wait(KFULL(gk % kKStages), (gk / kKStages) & 1)) { ok = false; break; }
-            tc::fence_after_sync();
-            issue_s(0, gk % kKStages);
-            issue_s(1, gk % kKStages);
-            tc::commit_warp(KEMPTY(gk % kKStages));
-            ++gk;
-            if (n == 1) tc::commit_warp(QEMPTY);
-            for (int j = 0; j < n; ++j) {
-                const int T = t + j, vst = gv % kVStages;
-                if (j == n - 1 && tail) {
-                    if (!wait(VZERO, nfix & 1)) { ok = false; break; }
-                } else if (!wait(VFULL(vst), (gv / kVStages) & 1)) {
-                    ok = false;
-                    break;
-                }
-                // O_0 += P_0(j) V(j), then S_0(j + 1)
-                if (!wait(PFULL(0), T & 1)) { ok = false; break; }
-                if (j == 0 && k >= 1 && !wait(OFREE(0), (k - 1) & 1)) { ok = false; break; }
-                tc::fence_after_sync();
-                issue_pv(0, vst, j > 0 ? 1u : 0u);
-                if (j == n - 1) tc::commit_warp(ODONE(0));
-                const bool more = j + 1 < n;
+#pragma unroll 1
+            for (int u = 0; u <= n; ++u) {
+                const int T = t + u - 1, vst = gv % kVStages, kst = gk % kKStages;
+                const uint32_t acc = u > 1 ? 1u : 0u;
                 // (one V stage: both P V first, so that the next V tile loads
                 // while both S of the next key tile run)
                 constexpr bool kPvFirst = Cfg::kVStages == 1;
-                if (!kPvFirst && more) {
-                    if (!wait(KFULL(gk % kKStages), (gk / kKStages) & 1)) { ok = false; break; }
+                if (u > 0) {
+                    if (u == n && tail) {
+                        if (!wait(VZERO, nfix & 1)) { ok = false; break; }
+                    } else if (!wait(VFULL(vst), (gv / kVStages) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    if (!wait(PFULL(0), T & 1)) { ok = false; break; }
+                    if (u == 1 && k >= 1 && !wait(OFREE(0), (k - 1) & 1)) { ok = false; break; }
                     tc::fence_after_sync();
-                    issue_s(0, gk % kKStages);
+                    issue_pv(0, vst, acc);
+                    if (u == n) tc::commit_warp(ODONE(0));
                 }
-                // O_1 += P_1(j) V(j), then S_1(j + 1)
-                if (!wait(PFULL(1), T & 1)) { ok = false; break; }
-                if (j == 0 && k >= 1 && !wait(OFREE(1), (k - 1) & 1)) { ok = false; break; }
-                tc::fence_after_sync();
-                issue_pv(1, vst, j > 0 ? 1u : 0u);
-                tc::commit_warp(VEMPTY(vst));
-                ++gv;
-                if (j == n - 1) tc::commit_warp(ODONE(1));
-                if (kPvFirst && more) {
-                    if (!wait(KFULL(gk % kKStages), (gk / kKStages) & 1)) { ok = false; break; }
+                if (!kPvFirst && u < n) {
+                    if (!wait(KFULL(kst), (gk / kKStages) & 1)) { ok = false; break; }
                     tc::fence_after_sync();
-                    issue_s(0, gk % kKStages);
+                    issue_s(0, kst);
                 }
-                if (more) {
-                    issue_s(1, gk % kKStages);
-                    tc::commit_warp(KEMPTY(gk % kKStages));
+                if (u > 0) {
+                    if (!wait(PFULL(1), T & 1)) { ok = false; break; }
+                    if (u == 1 && k >= 1 && !wait(OFREE(1), (k - 1) & 1)) { ok = false; break; }
+                    tc::fence_after_sync();
+                    issue_pv(1, vst, acc);
+                    tc::commit_warp(VEMPTY(vst));
+                    ++gv;
+                    if (u == n) tc::commit_warp(ODONE(1));
+                }
+                if (u < n) {
+                    if (kPvFirst) {
+                        if (!wait(KFULL(kst), (gk / kKStages) & 1)) { ok = false; break; }
+                        tc::fence_after_sync();
+                        issue_s(0, kst);
+                    }
+                    issue_s(1, kst);
+                    tc::commit_warp(KEMPTY(kst));
                     ++gk;
-                    if (j + 1 == n - 1) tc::commit_warp(QEMPTY);  // last S of this item
+                    if (u == n - 1) tc::commit_warp(QEMPTY);  // last S of this item
                 }
             }
             if (!ok) break;
@@ -578,7 +560,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 tc::tmem_wait_st();
                 tc::fence_before_sync();
-                tc::mbar_arrive(PFULL(w));
+                __syncwarp();
+                tc::mbar_arrive_warp(PFULL(w));
             }
             if (!ok) break;
             if (!wait(ODONE(w), k & 1)) break;
@@ -691,8 +674,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             t += it.ntiles;
             tc::fence_before_sync();
-            tc::mbar_arrive(OFREE(w));  // O_w may be overwritten by the next item
-            tc::mbar_arrive(ITEMEMPTY(slot));
+            __syncwarp();
+            tc::mbar_arrive_warp(OFREE(w));  // O_w may be overwritten by the next item
+            tc::mbar_arrive_warp(ITEMEMPTY(slot));
         }
     }
 

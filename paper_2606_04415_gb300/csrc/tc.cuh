@@ -226,10 +226,15 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint3
         "r"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
+// True in one lane of the (converged) warp: a burst of MMAs and their commit
+// goes into one branch on it, followed by __syncwarp().
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+    return ok != 0;
+}
 // Warp-collective forms: the whole warp executes them with uniform operands
-// and one elected lane issues the instruction. Keeping the issuing code
-// warp-uniform lets the operands stay in uniform registers, which is what
-// lets back-to-back MMAs issue at the tensor core's rate.
+// and one elected lane issues the instruction.
 __device__ __forceinline__ void mma_ts_warp(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n .reg .pred p, q;\n setp.ne.b32 q, %4, 0;\n elect.sync _|p, 0xffffffff;\n"
