@@ -42,10 +42,10 @@
 //   warps 6-9  the next item's tensor-memory part of Q (held in registers
 //              until the last S of the current item is done) and the epilogue
 //              of the last item, beside the next item's first S and softmax.
-// Measured, one 1024-token prompt and 256 decodes of 1024..16384 keys: 983 us a
-// step with one CTA per item and P over S's columns, 921 with this kernel in a
-// loop that lasts (at the power limit, SM clock 1785 of 2070 MHz), 847 in a
-// short one; the prompt alone 281 us and 206.
+// Measured, one 1024-token prompt and 256 decodes of 1024..16384 keys: 974 us a
+// step with one CTA per item and P over S's columns, 904 with this kernel in a
+// loop that lasts (at the power limit, SM clock 1785 of 2070 MHz), 839 in a
+// short one; the prompt alone 281 us and 208.
 // Every mbarrier wait is bounded; a timeout raises the plan's error flag and
 // the CTA drains its copies and tensor-core work, frees its tensor memory and
 // exits.
@@ -276,7 +276,8 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
         // warps run different code side by side, and an issuer with a copy
         // per half and for the first tile (150 unrolled MMAs) and the softmax
         // evicted each other from the instruction cache (2.7 us a tile; rolled
-        // loops over the chunks took 2.0 us by their address arithmetic). A
+        // loops over the chunks took 2.0 us by their address arithmetic). One
+        // elected lane issues a burst (electing one for each product cost 3%). A
         // wait costs this warp 100 to 170 cycles and a commit 80 to 120 with
         // the tensor pipe idle, so the softmax warps wait for the next tile's
         // V part (before they signal P) and free the first part's slots.
@@ -298,32 +299,40 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
                     if (u == 0 && !wait(VFULL(st), (gt / kStages) & 1)) { ok = false; break; }
                     if (gt > 0 && !wait(SFREE, (gt - 1) & 1)) { ok = false; break; }  // the tile before is in registers
                     tc::fence_after_sync();
+                    if (tc::elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < 4 * kQsChunks; ++kk)
-                        tc::mma_ss_warp(tS, qd + ((kk / 4) * kQChunkBytes + (kk % 4) * 32) / 16,
-                                        nd + ((kk / 4) * kChunkBytes + (kk % 4) * 32) / 16, idS, kk > 0 ? 1u : 0u);
+                        for (int kk = 0; kk < 4 * kQsChunks; ++kk)
+                            tc::mma_ss(tS, qd + ((kk / 4) * kQChunkBytes + (kk % 4) * 32) / 16,
+                                       nd + ((kk / 4) * kChunkBytes + (kk % 4) * 32) / 16, idS, kk > 0 ? 1u : 0u);
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)  // the rotary columns
-                        tc::mma_ts_warp(tS, tQ + 128 + kk * 8, nd + (4 * kChunkBytes + kk * 32) / 16, idS, 1u);
+                        for (int kk = 0; kk < 4; ++kk)  // the rotary columns
+                            tc::mma_ts(tS, tQ + 128 + kk * 8, nd + (4 * kChunkBytes + kk * 32) / 16, idS, 1u);
+                    }
+                    __syncwarp();
                     issued = true;
                 }
                 if (u > 0) {  // O += P(u - 1) V(u - 1)
                     if (!wait(PREADY, (gt - 1) & 1)) { ok = false; break; }
                     if (u == 1 && k >= 1 && !wait(OFREE, (k - 1) & 1)) { ok = false; break; }
                     tc::fence_after_sync();
-                    tc::mma_ts_warp(tO, tP, vd, idO, acc);
+                    if (tc::elect_one()) {
+                        tc::mma_ts(tO, tP, vd, idO, acc);
 #pragma unroll
-                    for (int kk = 1; kk < kKeysT / 16; ++kk)
-                        tc::mma_ts_warp(tO, tP + kk * 8, vd + (kk * 2048) / 16, idO, 1u);
-                    tc::commit_warp(VEMPTY(st ^ 1));
-                    if (u == n) tc::commit_warp(ODONE);
+                        for (int kk = 1; kk < kKeysT / 16; ++kk) tc::mma_ts(tO, tP + kk * 8, vd + (kk * 2048) / 16, idO, 1u);
+                        tc::commit(VEMPTY(st ^ 1));
+                        if (u == n) tc::commit(ODONE);
+                    }
+                    __syncwarp();
                 }
                 if (u < n) {  // S(u) over the chunks of this half's V
+                    if (tc::elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < 4 * kVChunks; ++kk)
-                        tc::mma_ts_warp(tS, tQ + kk * 8, kd + ((kk / 4) * kChunkBytes + (kk % 4) * 32) / 16, idS, 1u);
-                    tc::commit_warp(SFULL);
-                    if (u == n - 1) tc::commit_warp(QFREE);  // the last S of this item
+                        for (int kk = 0; kk < 4 * kVChunks; ++kk)
+                            tc::mma_ts(tS, tQ + kk * 8, kd + ((kk / 4) * kChunkBytes + (kk % 4) * 32) / 16, idS, 1u);
+                        tc::commit(SFULL);
+                        if (u == n - 1) tc::commit(QFREE);  // the last S of this item
+                    }
+                    __syncwarp();
                     ++gt;
                 }
             }
