@@ -74,6 +74,7 @@ struct fnpu_plan {
     float *d_ppart_lse = nullptr;
     float *d_ppart_o = nullptr;
     int32_t num_pparts = 0, num_pgroups = 0;
+    int32_t pitems_dual = 0;  // prefill items of one Q tile on both softmax paths
     // co-location (Sec. 3.4): prefill CTAs on pre_ctas SMs and decode CTAs on
     // the others, launched on two library streams forked from and joined back
     // into the caller's stream; e_started fires once all prefill CTAs began
@@ -247,8 +248,10 @@ int32_t choose_decode_sms(const std::vector<int64_t> &item_tiles, double tile_sc
 // range is split.
 struct TcUnit {
     int32_t seq, kvh, r0, rows;
-    int32_t ntiles;     // 64-key tiles its rows can see
-    int32_t max_start;  // last tile a split may start at: every row must see a key of every split
+    int32_t ntiles;     // steps: 128-key tiles its rows can see, pairs of them for a single Q tile
+    int32_t max_start;  // last step a split may start at: every row must see a key of every split
+    int32_t dual;       // the rows fill one Q tile at most: two key tiles a step, merged at the end
+    int32_t ktiles;     // 128-key tiles
 };
 
 // Cost model of a prefill work item in units of one 128-key tile of both Q
@@ -256,6 +259,12 @@ struct TcUnit {
 // for a split item, writing its partial result and the merge.
 constexpr int64_t kTcItemCost = 2;
 constexpr int64_t kTcMergeCost = 4;
+constexpr int64_t kTcDualMergeCost = 1;
+// A chunk of at most one Q tile takes two key tiles a step from this many on
+// (the exchange of the two paths costs about one tile). The short last item of a
+// longer chunk does not: beside full items it is over early either way, and four
+// chunks of 512 tokens took 39.7 us with it against 34.5.
+constexpr int32_t kDualTiles = 4;
 
 // First tile of split j of n over ntiles tiles (split n is the end).
 int32_t split_bound(int32_t ntiles, int32_t n, int32_t j) {
@@ -348,6 +357,19 @@ std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, int
     }
     std::vector<int64_t> caps = {maxc};
     for (int k = 2; k <= 8; ++k) caps.push_back((maxc + k - 1) / k);
+    // (units of one Q tile: a wave of them ends with its longest, so caps just
+    // below it are tried as well: 32 sequences of 4 tokens on 700..5000 keys
+    // 55.2 us a step without them (192 items), 45.9 with (160))
+    // Their splits hold one Q tile and merge in less time (a sequence of 4
+    // tokens on 2000 keys 23.7 us a step whole, 20.8 in two).
+    bool dual = false, all_dual = !units.empty();
+    for (const TcUnit &u : units) {
+        dual |= u.dual != 0;
+        all_dual &= u.dual != 0;
+    }
+    const int64_t merge_cost = all_dual ? kTcDualMergeCost : kTcMergeCost;
+    if (dual)
+        for (int k = 9; k <= 15; ++k) caps.push_back((maxc * k + 15) / 16);
     // (cap below: pieces shorter than 4 tiles cost more than they balance)
     for (int j = 1; j <= 8; ++j) caps.push_back((total + static_cast<int64_t>(sms) * j - 1) / (static_cast<int64_t>(sms) * j));
     std::vector<int32_t> best(units.size(), 1), ns(units.size(), 1);
@@ -358,7 +380,7 @@ std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, int
             if (std::find(uniq.begin(), uniq.end(), c) == uniq.end()) uniq.push_back(c);
         caps.swap(uniq);
     }
-    std::vector<int32_t> hist(static_cast<size_t>(maxc + kTcItemCost + kTcMergeCost) + 1);
+    std::vector<int32_t> hist(static_cast<size_t>(maxc + kTcItemCost + merge_cost) + 1);
     // the most splits a unit can take (at most 16): its last split must start
     // at or before max_start, and that start, floor(ntiles (n - 1) / n), does
     // not decrease with n, so the feasible counts are 1 .. nmax
@@ -370,7 +392,7 @@ std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, int
     }
     // split_units[c]: units longer than c tiles that may split. Under a cap
     // of c exactly these split, each into two pieces or more, and a unit cut
-    // into n >= 2 pieces costs at least kTcItemCost + 2 kTcMergeCost more than
+    // into n >= 2 pieces costs at least kTcItemCost + 2 merge_cost more than
     // whole; with the total of the unsplit items that bounds a candidate's
     // total from below before its splits are worked out
     std::vector<int32_t> split_units(static_cast<size_t>(maxc) + 2, 0);
@@ -384,7 +406,7 @@ std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, int
         if (best_span >= 0) {
             const int64_t nsplit = cap >= maxc ? 0 : split_units[static_cast<size_t>(cap)];
             if (nsplit == 0) continue;  // no unit splits: the first candidate's items
-            const int64_t lb = whole + nsplit * (kTcItemCost + 2 * kTcMergeCost);
+            const int64_t lb = whole + nsplit * (kTcItemCost + 2 * merge_cost);
             if ((lb + sms - 1) / sms >= best_span) continue;
         }
         // ceil(ntiles / cap) = floor((ntiles - 1) / cap) + 1 in double, exact
@@ -406,7 +428,7 @@ std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, int
                 n = std::min(q, nmax[i]);
             }
             ns[i] = n;
-            tot += units[i].ntiles + static_cast<int64_t>(n) * (kTcItemCost + (n > 1 ? kTcMergeCost : 0));
+            tot += units[i].ntiles + static_cast<int64_t>(n) * (kTcItemCost + (n > 1 ? merge_cost : 0));
         }
         if (ns == prev) continue;  // the same splits as the candidate before
         prev = ns;
@@ -416,7 +438,7 @@ std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, int
             // n pieces of floor(ntiles / n) or one more tiles (split_bound
             // rounds down), the longer ones ntiles mod n of them
             const int32_t n = ns[i], nt = units[i].ntiles, q = nt / n, r = nt % n;
-            const int32_t extra = kTcItemCost + (n > 1 ? kTcMergeCost : 0);
+            const int32_t extra = kTcItemCost + (n > 1 ? merge_cost : 0);
             hist[static_cast<size_t>(q + 1 + extra)] += r;
             hist[static_cast<size_t>(q + extra)] += n - r;
         }
@@ -853,8 +875,10 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
             for (int32_t r0 = 0; r0 < q; r0 += P2) {
                 const int32_t rows = std::min(P2, q - r0);
                 const int32_t ntiles = (prefix + r0 + rows + KT - 1) / KT;
+                const bool dual = q <= P2 / 2 && ntiles >= kDualTiles && desc->head_dim_qk == desc->head_dim_v;
+                const int32_t per = dual ? 2 : 1;
                 for (int32_t kvh = 0; kvh < desc->num_kv_heads; ++kvh)
-                    tc_units.push_back(TcUnit{s, kvh, r0, rows, ntiles, (prefix + r0) / KT});
+                    tc_units.push_back(TcUnit{s, kvh, r0, rows, (ntiles + per - 1) / per, (prefix + r0) / KT / per, dual, ntiles});
             }
         } else {
             const int32_t prefix = c - q;
@@ -939,6 +963,7 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
         }
     }
     int32_t pparts = 0, pgroups = 0;
+    pl->pitems_dual = 0;
     if (!tc_units.empty()) {
         const std::vector<int32_t> ns = choose_prefill_splits(tc_units, pl->pre_ctas);
         for (size_t u = 0; u < tc_units.size(); ++u) {
@@ -949,13 +974,15 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
                 pparts += n;
                 pgroups += 1;
             }
+            const int32_t per = t.dual ? 2 : 1;
+            pl->pitems_dual |= t.dual;
             for (int32_t j = 0; j < n; ++j) {
                 const int32_t kb = split_bound(t.ntiles, n, j), ke = split_bound(t.ntiles, n, j + 1);
                 pcost.emplace_back(static_cast<int64_t>(ke - kb) + kTcItemCost + (n > 1 ? kTcMergeCost : 0),
                                    static_cast<int32_t>(pitems.size()));
-                pitems.push_back(PrefillItem{t.seq, t.kvh, t.r0, t.rows, kb, ke, j, n, base, grp,
+                pitems.push_back(PrefillItem{t.seq, t.kvh, t.r0, t.rows, per * kb, std::min(per * ke, t.ktiles), j, n, base, grp,
                                              seqs[t.seq].q_start, seqs[t.seq].ctx_len - seqs[t.seq].q_len,
-                                             seqs[t.seq].ctx_len, seqs[t.seq].bt_row, 0, 0});
+                                             seqs[t.seq].ctx_len, seqs[t.seq].bt_row, t.dual, 0});
             }
         }
     }
@@ -1268,6 +1295,7 @@ AttnParams run_params(const fnpu_plan *pl, const void *q, const void *k_cache, c
     p.counters = pl->d_counters;
     p.pitems = pl->d_pitems;
     p.num_pitems = pl->num_pitems;
+    p.pitems_dual = pl->pitems_dual;
     p.ppart_o = pl->d_ppart_o;
     p.ppart_lse = pl->d_ppart_lse;
     p.pcounters = pl->d_pcounters;

@@ -37,7 +37,8 @@ struct PrefillItem {
     int32_t kt_begin, kt_end, split, num_splits;
     int32_t part_base, group;
     int32_t q_start, prefix, ctx_len, bt_row;  // the sequence's SeqInfo, so one load decodes an item
-    int32_t pad0, pad1;
+    int32_t dual;  // tcgen05 path: at most one Q tile of rows, its key tiles alternate between the two softmax paths
+    int32_t pad0;
 };
 static_assert(sizeof(PrefillItem) == 64, "PrefillItem layout");
 
@@ -96,6 +97,7 @@ struct AttnParams {
     // prefill
     const PrefillItem *pitems;
     int32_t num_pitems;
+    int32_t pitems_dual;    // some of them have `dual` set
     float *ppart_o;         // fp32 split-prefill partials, per partial: [2 tiles][dv / 4][128 rows] float4
     float *ppart_lse;       // fp32 [num_pparts, 2, 128] (log2 domain)
     int32_t *pcounters;     // [num_pgroups, 8] one per softmax warp, zero between runs

@@ -12,6 +12,11 @@
 // head (2P positions) that consume the same K/V tiles, which halves the
 // L2-to-SM traffic per FLOP.
 //
+// An item of one Q tile only (a few tokens of a decode verified at once, the
+// end of a chunk) puts the same Q tile on both paths, with the even key tiles
+// on one and the odd ones on the other, and merges the two results from tensor
+// memory: without it half of the tensor and softmax work went to an empty tile.
+//
 // Key tiles are 128 keys wide: an S = Q K^T product is then M = N = 128 and
 // runs at the full tensor rate (a 64-wide one, with both operands in shared
 // memory, is bound by shared-memory bandwidth: 48 instead of 32 cycles).
@@ -87,9 +92,10 @@ struct TcCfg {
     static constexpr int kQOff = kVOff + kVStages * kVTileBytes;
     static constexpr int kBarOff = kQOff + 2 * kQBytes;
     // kfull[3] kempty[3] vfull[2] vempty[2] sfull[2] pfull[2] odone[2] ofree[2]
-    // qfull qempty vzero itemfull[2] itemempty[2] drain
-    static constexpr int kNumBars = 2 * kKStages + 2 * kVStages + 8 + 3 + 4 + 1;
-    static constexpr int kSmemUsed = kBarOff + 8 * kNumBars + 32;
+    // qfull qempty vzero itemfull[2] itemempty[2] drain mlx oread
+    static constexpr int kNumBars = 2 * kKStages + 2 * kVStages + 8 + 3 + 4 + 3;
+    static constexpr int kMlOff = kBarOff + 8 * kNumBars + 32;  // (m, l) of both paths' rows (dual items)
+    static constexpr int kSmemUsed = kMlOff + 2 * 128 * 8;
     // at least 116 KB so that no two CTAs share an SM (each holds all 512 TMEM columns)
     static constexpr int kSmemBytes = kSmemUsed > 116 * 1024 ? kSmemUsed : 116 * 1024;
     static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
@@ -99,15 +105,19 @@ struct TcMaps {
     CUtensorMap k, v, q;
 };
 
-struct ItemGeom {
+// dual: one Q tile, its even key tiles on tile 0's path and its odd ones on tile 1's
+template <bool kDual>
+struct ItemGeomT {
     int kvh, p0, rows, prefix, ctx, kt0, ntiles, q_start, bt_row;
     int ns, split, pbase, cnt;  // key splits of the tile pair, this split, first partial, merge counter
     bool tail_fix;
+    bool dual;
 };
 
-__device__ __forceinline__ ItemGeom item_geom(const AttnParams &p, int idx) {
+template <bool kDual>
+__device__ __forceinline__ ItemGeomT<kDual> item_geom(const AttnParams &p, int idx) {
     const PrefillItem it = p.pitems[idx];  // carries its sequence's fields: one load
-    ItemGeom g;
+    ItemGeomT<kDual> g;
     g.kvh = it.head;
     g.p0 = it.row_begin;
     g.rows = it.rows;
@@ -122,6 +132,7 @@ __device__ __forceinline__ ItemGeom item_geom(const AttnParams &p, int idx) {
     g.pbase = it.part_base;
     g.cnt = it.group;
     g.tail_fix = it.kt_end * kKeys > g.ctx;
+    g.dual = kDual && it.dual != 0;
     return g;
 }
 
@@ -133,7 +144,7 @@ __device__ __forceinline__ ItemGeom item_geom(const AttnParams &p, int idx) {
 // cooperative, so all are resident. False if the wait ran out (the plan's
 // error flag is raised). A call of its own, so that the kernel's warps keep
 // their register allocation.
-__device__ __noinline__ bool fused_append(const AttnParams &p, int tid) {
+__device__ __noinline__ bool fused_append(const AttnParams &p, int tid, volatile int *ok_all) {
     const int32_t kc = p.fa_k_chunks, per_tok = kc + p.fa_v_chunks;
     const int64_t total = static_cast<int64_t>(p.fa_num_tokens) * per_tok;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + tid; i < total;
@@ -153,7 +164,6 @@ __device__ __noinline__ bool fused_append(const AttnParams &p, int tid) {
     }
     tc::fence_proxy_async_global();  // before the TMA reads of the rows, here and in other CTAs
     __syncthreads();
-    __shared__ int ok_all;
     if (tid == 0) {
         __threadfence();
         atomicAdd(p.fa_count, 1);
@@ -167,15 +177,17 @@ __device__ __noinline__ bool fused_append(const AttnParams &p, int tid) {
             __nanosleep(32);
         }
         tc::fence_proxy_async_global();
-        ok_all = ok;
+        *ok_all = ok;
     }
     __syncthreads();
-    return ok_all != 0;
+    return *ok_all != 0;
 }
 
 // F16: the operands (Q, K, V and P) are f16 instead of bf16 (the FP8 cache's
 // prefill: its codes are dequantised to f16 first)
-template <int DQ, int DV, bool F16>
+// kDual: the plan has items of a single Q tile on both paths (a kernel of its
+// own: the code for them costs the others 2 to 4% through the instruction cache)
+template <int DQ, int DV, bool F16, bool kDual>
 __global__ void __launch_bounds__(kThreads, 1)
     prefill_tc_kernel(const AttnParams p, const __grid_constant__ TcMaps maps) {
     using Cfg = TcCfg<DQ, DV>;
@@ -195,11 +207,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t QFULL = b0 + 64, QEMPTY = b0 + 72, VZERO = b0 + 80;
     auto ITEMFULL = [&](int k) { return b0 + 88 + 8 * k; };
     auto ITEMEMPTY = [&](int k) { return b0 + 104 + 8 * k; };
-    const uint32_t DRAIN = b0 + 120;
+    const uint32_t DRAIN = b0 + 120, MLX = b0 + 128, OREAD = b0 + 136;
+    float2 *ml = reinterpret_cast<float2 *>(smem + Cfg::kMlOff);
     uint8_t *misc = smem + Cfg::kBarOff + 8 * Cfg::kNumBars;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(misc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 4);
-    volatile int *item_slot = reinterpret_cast<volatile int *>(misc + 8);  // [2]
+    volatile int *item_slot = reinterpret_cast<volatile int *>(misc + 8);  // [2], then the fused append's result
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = p.group;
@@ -230,6 +243,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::mbar_init(QEMPTY, 1);
         tc::mbar_init(VZERO, 1);
         tc::mbar_init(DRAIN, 1);
+        if (kDual) {
+            tc::mbar_init(MLX, 8);  // the softmax warps of both paths
+            tc::mbar_init(OREAD, 8);
+        }
         *abort_flag = 0;
         tc::fence_mbar_init();
     }
@@ -241,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
 
-    if (p.fa_count != nullptr && !fused_append(p, tid)) *abort_flag = 1;
+    if (p.fa_count != nullptr && !fused_append(p, tid, item_slot + 2)) *abort_flag = 1;
 
     auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
         if (tc::mbar_try_wait(bar, parity)) return true;
@@ -288,12 +305,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 idx = __shfl_sync(0xffffffffu, item_slot[slot], 0);
                 if (idx < 0) break;
             }
-            const ItemGeom it = item_geom(p, idx);
+            const ItemGeomT<kDual> it = item_geom<kDual>(p, idx);
             const int ukvh = __shfl_sync(0xffffffffu, it.kvh, 0);
             // both Q tiles, once the previous item's last S is done (loading them
             // after the item's first K tiles, with an L2 prefetch ahead, was
             // measured slower)
             const int q0 = __shfl_sync(0xffffffffu, it.q_start + it.p0, 0);
+            const int q_step = kDual ? __shfl_sync(0xffffffffu, it.dual ? 0 : P, 0) : P;
             auto load_q = [&]() -> bool {
                 if (k >= 1 && !wait(QEMPTY, (k - 1) & 1)) return false;
                 tc::mbar_arrive_expect_tx_warp(QFULL, static_cast<uint32_t>(2 * (DQ / 64) * 64 * G * P * 2));
@@ -302,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                     for (int h = 0; h < DQ / 64; ++h)
                         tc::tma_load_3d_warp(s_base + Cfg::kQOff + w * Cfg::kQBytes + h * Cfg::kQHalf, &maps.q,
-                                             QFULL, h * 64, ukvh * G, q0 + w * P);
+                                             QFULL, h * 64, ukvh * G, q0 + w * q_step);
                 return true;
             };
             const int32_t *bt = p.block_table + static_cast<int64_t>(it.bt_row) * p.bt_stride;
@@ -364,7 +382,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         constexpr uint32_t idO = F16 ? tc::idesc_f16(kRows, DV, true) : tc::idesc_bf16(kRows, DV, true);
         const uint32_t utmem = __shfl_sync(0xffffffffu, tmem, 0);
         const uint32_t us_base = __shfl_sync(0xffffffffu, s_base, 0);
-        int gk = 0, gv = 0, t = 0, nfix = 0;
+        int gk = 0, gv = 0, t0 = 0, t1 = 0, nfix = 0;  // ring positions, tiles done by each Q tile
         bool ok = true, issued = false;
         auto issue_s = [&](int w, int st) {
             if (tc::elect_one()) {
@@ -396,16 +414,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!wait(ITEMFULL(slot), (k >> 1) & 1)) { ok = false; break; }
             const int idx = __shfl_sync(0xffffffffu, item_slot[slot], 0);
             if (idx < 0) break;
-            const ItemGeom it = item_geom(p, idx);
+            const ItemGeomT<kDual> it = item_geom<kDual>(p, idx);
             const int n = __shfl_sync(0xffffffffu, it.ntiles, 0);
             const bool tail = __shfl_sync(0xffffffffu, it.tail_fix ? 1 : 0, 0) != 0;
             // PV_0(u - 1), S_0(u), PV_1(u - 1), S_1(u) for u = 0 .. n: each product
             // has one place in the code, so that the issuer takes little of the
             // instruction cache that it shares with the softmax
             if (!wait(QFULL, k & 1)) { ok = false; break; }
+            const bool dual = kDual && __shfl_sync(0xffffffffu, it.dual ? 1 : 0, 0) != 0;
 #pragma unroll 1
-            for (int u = 0; u <= n; ++u) {
-                const int T = t + u - 1, vst = gv % kVStages, kst = gk % kKStages;
+            for (int u = 0; !dual && u <= n; ++u) {
+                const int T = t0 + u - 1, vst = gv % kVStages, kst = gk % kKStages;
                 const uint32_t acc = u > 1 ? 1u : 0u;
                 // (one V stage: both P V first, so that the next V tile loads
                 // while both S of the next key tile run)
@@ -429,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     issue_s(0, kst);
                 }
                 if (u > 0) {
-                    if (!wait(PFULL(1), T & 1)) { ok = false; break; }
+                    if (!wait(PFULL(1), (kDual ? t1 + u - 1 : T) & 1)) { ok = false; break; }
                     if (u == 1 && k >= 1 && !wait(OFREE(1), (k - 1) & 1)) { ok = false; break; }
                     tc::fence_after_sync();
                     issue_pv(1, vst, acc);
@@ -449,8 +468,43 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (u == n - 1) tc::commit_warp(QEMPTY);  // last S of this item
                 }
             }
+            // one Q tile on both paths: path w takes key tiles w, w + 2, ... with a
+            // K and a V slot of its own for each
+#pragma unroll 1
+            for (int u = 0; kDual && dual && u <= (n + 1) / 2; ++u) {
+#pragma unroll 1
+                for (int w = 0; ok && w < 2; ++w) {
+                    const int nw = (n + 1 - w) / 2;
+                    if (u > 0 && u <= nw) {
+                        const int vst = gv % kVStages;
+                        const bool fix = tail && 2 * (u - 1) + w == n - 1;
+                        if (!wait(fix ? VZERO : VFULL(vst), fix ? nfix & 1 : (gv / kVStages) & 1) ||
+                            !wait(PFULL(w), ((w ? t1 : t0) + u - 1) & 1) ||
+                            (u == 1 && k >= 1 && !wait(OFREE(w), (k - 1) & 1))) {
+                            ok = false;
+                            break;
+                        }
+                        tc::fence_after_sync();
+                        issue_pv(w, vst, u > 1 ? 1u : 0u);
+                        tc::commit_warp(VEMPTY(vst));
+                        ++gv;
+                    }
+                    if (u == nw) tc::commit_warp(ODONE(w));
+                    if (u < nw) {
+                        const int kst = gk % kKStages;
+                        if (!wait(KFULL(kst), (gk / kKStages) & 1)) { ok = false; break; }
+                        tc::fence_after_sync();
+                        issue_s(w, kst);
+                        tc::commit_warp(KEMPTY(kst));
+                        ++gk;
+                        if (2 * u + w == n - 1) tc::commit_warp(QEMPTY);  // last S of this item
+                    }
+                }
+                if (!ok) break;
+            }
             if (!ok) break;
-            t += n;
+            t0 += dual ? (n + 1) / 2 : n;
+            if (kDual) t1 += dual ? n / 2 : n;
             if (tail) ++nfix;
             tc::mbar_arrive_warp(ITEMEMPTY(slot));
         }
@@ -467,14 +521,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const int pl = r / G, hl = r % G;
         const float sc = p.scale_log2;
-        int t = 0;
+        int t = 0, nd = 0;  // tiles of this path and dual items so far
         for (int k = 0;; ++k) {
             const int slot = k & 1;
             if (!wait(ITEMFULL(slot), (k >> 1) & 1)) break;
             const int idx = item_slot[slot];
             if (idx < 0) break;
-            const ItemGeom it = item_geom(p, idx);
-            const int pw = it.p0 + w * P;
+            const ItemGeomT<kDual> it = item_geom<kDual>(p, idx);
+            const int pw = it.p0 + (kDual && it.dual ? 0 : w * P);
+            const int nw = kDual && it.dual ? (it.ntiles + 1 - w) / 2 : it.ntiles;  // key tiles of this path
             const bool row_ok = (r < P * G) && (pw + pl < it.p0 + it.rows);
             // rows past the item (padding) keep a position too; their results are
             // never stored, so they need no masking of their own
@@ -486,7 +541,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             float m_run = -INFINITY;  // reference max (log2 units) of the exponentials
             float l = 0.f;
             bool ok = true;
-            for (int i = 0; i < it.ntiles; ++i) {
+            for (int i = 0; i < nw; ++i) {
                 const int T = t + i;
                 if (!wait(SFULL(w), T & 1)) { ok = false; break; }
                 tc::fence_after_sync();
@@ -497,7 +552,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tc::tmem_wait_ld();
                 // tiles that reach past the first row's position need the causal
                 // mask; all others are fully visible to every row of the tile
-                const int k0 = (it.kt0 + i) * kKeys;
+                const int k0 = (it.kt0 + (kDual && it.dual ? 2 * i + w : i)) * kKeys;
                 const bool masked_tile = k0 + kKeys - 1 > min_pos;
                 if (masked_tile) {
 #pragma unroll
@@ -566,10 +621,110 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!ok) break;
             if (!wait(ODONE(w), k & 1)) break;
             tc::fence_after_sync();
-            const float inv = 1.f / l;
             uint4 *orow = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(p.out) +
                                                     (tok * p.num_q_heads + head) * DV);
-            if (it.ns == 1) {
+            const float inv = 1.f / l;  // (a dual item's row may see no key on one path; it has its own sums)
+            if (kDual && it.dual) {
+                // One Q tile on both paths: each path has the row's maximum and
+                // sum over its key tiles, and both O are in tensor memory, same
+                // lane. The paths exchange (m, l) and write half of the columns
+                // each: out = (O_0 2^(m0 - M) + O_1 2^(m1 - M)) / L.
+                ml[w * 128 + r] = make_float2(m_run, l);
+                __syncwarp();
+                tc::mbar_arrive_warp(MLX);
+                if (!wait(MLX, nd & 1) || !wait(ODONE(1 - w), k & 1)) break;
+                tc::fence_after_sync();
+                const float2 a = ml[r], b = ml[128 + r];
+                const bool va = a.y > 0.f, vb = b.y > 0.f;
+                const float M = fmaxf(va ? a.x : -INFINITY, vb ? b.x : -INFINITY);
+                const float fa = va ? fast_exp2(a.x - M) : 0.f, fb = vb ? fast_exp2(b.x - M) : 0.f;
+                const float L = a.y * fa + b.y * fb, iL = 1.f / L;
+                const float ca = fa * iL, cb = fb * iL;
+                const int64_t prow = (static_cast<int64_t>(it.pbase + it.split) * 2) * 128;
+                float4 *po = reinterpret_cast<float4 *>(p.ppart_o) + prow * (DV / 4) + r;
+#pragma unroll 1
+                for (int c = w * (DV / 64); c < (w + 1) * (DV / 64); ++c) {
+                    uint32_t o0[32], o1[32];
+                    tc::tmem_ld32(lane_addr + col_o(0) + 32 * c, o0);
+                    tc::tmem_ld32(lane_addr + col_o(1) + 32 * c, o1);
+                    tc::tmem_wait_ld();
+                    float v[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        v[j] = (va ? __uint_as_float(o0[j]) * ca : 0.f) + (vb ? __uint_as_float(o1[j]) * cb : 0.f);
+                    if (it.ns == 1) {
+                        if (row_ok) {
+#pragma unroll
+                            for (int j = 0; j < 2; ++j) {
+                                uint32_t x[8];
+#pragma unroll
+                                for (int y = 0; y < 8; ++y) x[y] = pack_bf16x2(v[16 * j + 2 * y], v[16 * j + 2 * y + 1]);
+                                st_global_v8(orow + c * 4 + 2 * j, x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            po[(c * 8 + j) * 128] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    }
+                }
+                const float my_lse = M + log2f(L);
+                if (it.ns == 1) {
+                    if (w == 0 && row_ok) p.lse[tok * p.num_q_heads + head] = my_lse * kLn2;
+                } else {
+                    // the last split to finish merges, each warp its rows and columns
+                    p.ppart_lse[prow + w * 128 + r] = my_lse;
+                    __threadfence();
+                    __syncwarp();
+                    int last = 0;
+                    if (lane == 0) last = atomicAdd(p.pcounters + it.cnt * 8 + (warp & 7), 1) == it.ns - 1;
+                    last = __shfl_sync(0xffffffffu, last, 0);
+                    if (last) {
+                        __threadfence();
+                        const int64_t row0 = static_cast<int64_t>(it.pbase) * 2 * 128;
+                        auto lse_of = [&](int sp) { return __ldcg(p.ppart_lse + row0 + sp * 256 + w * 128 + r); };
+                        float MM = -INFINITY, LL = 0.f;
+                        for (int sp = 0; sp < it.ns; ++sp) MM = fmaxf(MM, lse_of(sp));
+                        for (int sp = 0; sp < it.ns; ++sp) LL += fast_exp2(lse_of(sp) - MM);
+                        const float iLL = 1.f / LL;
+#pragma unroll 1
+                        for (int c = w * (DV / 64); c < (w + 1) * (DV / 64); ++c) {
+                            float4 acc[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            for (int sp = 0; sp < it.ns; ++sp) {  // in split order: reproducible
+                                const float ws = fast_exp2(lse_of(sp) - MM);
+                                const float4 *q4 = reinterpret_cast<const float4 *>(p.ppart_o) + (row0 + sp * 256) * (DV / 4) + r;
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) {
+                                    const float4 x = __ldcg(q4 + (c * 8 + j) * 128);
+                                    acc[j].x += ws * x.x; acc[j].y += ws * x.y;
+                                    acc[j].z += ws * x.z; acc[j].w += ws * x.w;
+                                }
+                            }
+                            if (row_ok) {
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    uint4 v;
+                                    v.x = pack_bf16x2(acc[2 * j].x * iLL, acc[2 * j].y * iLL);
+                                    v.y = pack_bf16x2(acc[2 * j].z * iLL, acc[2 * j].w * iLL);
+                                    v.z = pack_bf16x2(acc[2 * j + 1].x * iLL, acc[2 * j + 1].y * iLL);
+                                    v.w = pack_bf16x2(acc[2 * j + 1].z * iLL, acc[2 * j + 1].w * iLL);
+                                    orow[c * 4 + j] = v;
+                                }
+                            }
+                        }
+                        if (w == 0 && row_ok) p.lse[tok * p.num_q_heads + head] = (MM + log2f(LL)) * kLn2;
+                        if (lane == 0) p.pcounters[it.cnt * 8 + (warp & 7)] = 0;  // ready for the next run
+                    }
+                }
+                // both O are read by both paths before either is free
+                tc::fence_before_sync();
+                __syncwarp();
+                tc::mbar_arrive_warp(OREAD);
+                if (!wait(OREAD, nd & 1)) break;
+                ++nd;
+            } else if (it.ns == 1) {
 #pragma unroll
                 for (int c = 0; c < DV / 32; ++c) {
                     uint32_t o[32];
@@ -672,7 +827,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (lane == 0) p.pcounters[it.cnt * 8 + (warp & 7)] = 0;  // ready for the next run
                 }
             }
-            t += it.ntiles;
+            t += nw;
             tc::fence_before_sync();
             __syncwarp();
             tc::mbar_arrive_warp(OFREE(w));  // O_w may be overwritten by the next item
@@ -729,7 +884,7 @@ bool encode_q_map(CUtensorMap *m, const void *base, int d, int hq, int64_t T, in
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int DQ, int DV, bool F16>
+template <int DQ, int DV, bool F16, bool kDual>
 int launch_tc(const AttnParams &p, cudaStream_t st, int max_ctas, cudaEvent_t started, bool pdl) {
     using Cfg = TcCfg<DQ, DV>;
     TcMaps maps;
@@ -737,7 +892,7 @@ int launch_tc(const AttnParams &p, cudaStream_t st, int max_ctas, cudaEvent_t st
         !encode_cache_map(&maps.v, p.v_cache, DV, p.num_kv_heads, p.block_size, p.num_blocks, F16) ||
         !encode_q_map(&maps.q, p.q, DQ, p.num_q_heads, p.num_tokens, p.group, kRows / p.group, F16))
         return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");
-    auto kernel = prefill_tc_kernel<DQ, DV, F16>;
+    auto kernel = prefill_tc_kernel<DQ, DV, F16, kDual>;
     FNPU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
     FNPU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        cudaSharedmemCarveoutMaxShared));
@@ -766,14 +921,19 @@ int launch_prefill_tc(const AttnParams &p, void *stream, int max_ctas, void *sta
     if (p.num_pitems == 0) return FNPU_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaEvent_t ev = static_cast<cudaEvent_t>(started);
-    if (f16)
-        return p.head_dim_qk == 128 && p.head_dim_v == 128 ? launch_tc<128, 128, true>(p, st, max_ctas, ev, pdl)
-                                                            : FNPU_EUNSUPPORTED;
-    if (p.head_dim_qk == 64 && p.head_dim_v == 64) return launch_tc<64, 64, false>(p, st, max_ctas, ev, pdl);
+    const bool dual = p.pitems_dual != 0;
+    if (f16) {
+        if (p.head_dim_qk != 128 || p.head_dim_v != 128) return FNPU_EUNSUPPORTED;
+        return dual ? launch_tc<128, 128, true, true>(p, st, max_ctas, ev, pdl)
+                    : launch_tc<128, 128, true, false>(p, st, max_ctas, ev, pdl);
+    }
+    if (p.head_dim_qk == 64 && p.head_dim_v == 64)
+        return dual ? launch_tc<64, 64, false, true>(p, st, max_ctas, ev, pdl)
+                    : launch_tc<64, 64, false, false>(p, st, max_ctas, ev, pdl);
     if (p.head_dim_qk == 128 && p.head_dim_v == 128)
-        return launch_tc<128, 128, false>(p, st, max_ctas, ev, pdl);
-    if (p.head_dim_qk == 192 && p.head_dim_v == 128)
-        return launch_tc<192, 128, false>(p, st, max_ctas, ev, pdl);
+        return dual ? launch_tc<128, 128, false, true>(p, st, max_ctas, ev, pdl)
+                    : launch_tc<128, 128, false, false>(p, st, max_ctas, ev, pdl);
+    if (p.head_dim_qk == 192 && p.head_dim_v == 128) return launch_tc<192, 128, false, false>(p, st, max_ctas, ev, pdl);
     return FNPU_EUNSUPPORTED;
 }
 

@@ -303,6 +303,29 @@ def test_prefill_key_splits(bs, dim):
     assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
 
 
+@pytest.mark.parametrize("heads,dim,bs", [((28, 4), 128, 16), ((8, 2), 128, 64), ((4, 2), 64, 16), ((6, 6), 128, 32)])
+def test_single_q_tile_items(heads, dim, bs):
+    """Chunks of at most one Q tile, whose key tiles alternate between the two
+    softmax paths: even and odd tile counts around the line where that begins,
+    last tiles that few rows (or one) can see, one row more than a tile, and a
+    context long enough for key splits on top."""
+    hq, hkv = heads
+    P = 128 // (hq // hkv)  # positions of a Q tile
+    sh = W.Shape(hq, hkv, dim, dim, bs, False)
+    ctx = [384, 385, 512, 513, 514, 640, 641, 769, 1030, 9000]
+    for q in (2, P, P + 1):
+        rng = np.random.default_rng(q + hq)
+        ql = [min(q, c) for c in ctx]
+        batch = W.build_batch(sh, ql, ctx, [1] * len(ctx), rng, name="one_tile")
+        st = _step(batch)
+        out, lse = st.results()
+        tokens = None if q < 40 else _sample_tokens(batch, per_seq_rows=10)
+        _compare(batch, out, lse, tokens=tokens)
+        st.run()
+        out2, lse2 = st.results()
+        assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
+
+
 SEPARATE = 1  # FNPU_PLAN_SEPARATE_LAUNCHES
 
 
