@@ -517,15 +517,18 @@ namespace fnpu {
 namespace {
 // The tcgen05 prefill launch; over the FP8 cache, first the f16 staging of
 // the prefill sequences' blocks and of the queries, and the prefill reads those.
-// With pdl a bf16 prefill grid is a programmatic dependent launch of the
+// With pdl the first of these grids is a programmatic dependent launch of the
 // kernel before it on `stream` (the step's append): its CTAs set up while that
-// kernel drains, and its loaders wait for it before the first read.
+// kernel drains, and its loaders wait for it before the first read; and so is the
+// prefill of the staging, unless `started` is asked for (as the staging's
+// dependent, the prefill's launch-completion event held the decode beside it
+// back by some 65 us).
 int launch_prefill(const fnpu_plan *pl, const AttnParams &p, void *stream, int ctas, void *started,
                    bool pdl = false) {
     if (p.num_pitems == 0) return FNPU_OK;  // (nothing to stage either)
     if (!pl->desc.kv_fp8) return launch_prefill_tc(p, stream, ctas, started, false, pdl);
     const int rc = launch_fp8_stage(p.k_cache, p.v_cache, pl->d_jobs, pl->num_jobs, pl->d_tk, pl->d_tv, p.q, pl->d_tq,
-                                    p.num_tokens * p.num_q_heads * p.head_dim_qk, stream);
+                                    p.num_tokens * p.num_q_heads * p.head_dim_qk, stream, pdl);
     if (rc != FNPU_OK) return rc;
     AttnParams pp = p;
     pp.q = pl->d_tq;
@@ -534,7 +537,7 @@ int launch_prefill(const fnpu_plan *pl, const AttnParams &p, void *stream, int c
     pp.block_table = pl->d_tbt;
     pp.bt_stride = pl->tbt_width;
     pp.num_blocks = pl->num_tblocks;
-    return launch_prefill_tc(pp, stream, ctas, started, true);
+    return launch_prefill_tc(pp, stream, ctas, started, true, pdl && !started);
 }
 }  // namespace
 }  // namespace fnpu
@@ -1338,11 +1341,10 @@ int run_colocated(const fnpu_plan *pl, const AttnParams &p, void *stream) {
         // its CTAs take their SMs and set up while that kernel drains. The
         // decode stream waits for the fork (everything before the prefill is
         // done) and for the prefill grid's launch-completion event. (Over the
-        // FP8 cache the staging kernel comes before the prefill, which is then
-        // an ordinary launch: as the staging's dependent, the prefill's
-        // launch-completion event held the decode back by some 65 us.)
+        // FP8 cache the staging kernel comes before the prefill and is the one
+        // that follows the append so.)
         FNPU_CUDA_TRY(cudaStreamWaitEvent(pl->s_dec, pl->e_fork, 0));
-        int rc = launch_prefill(pl, p, s, pl->pre_ctas, pl->e_started, !pl->desc.kv_fp8);
+        int rc = launch_prefill(pl, p, s, pl->pre_ctas, pl->e_started, true);
         if (rc == FNPU_OK) {
             FNPU_CUDA_TRY(cudaStreamWaitEvent(pl->s_dec, pl->e_started, 0));
             rc = launch_decode(pl, p, pl->s_dec, 3 * pl->num_sms);

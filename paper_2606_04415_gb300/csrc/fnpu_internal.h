@@ -174,7 +174,7 @@ struct Fp8StageJob {
     int32_t dst, src, valid, pad;
 };
 int launch_fp8_stage(const void *k_pool, const void *v_pool, const Fp8StageJob *jobs, int32_t num_jobs, void *k_f16,
-                     void *v_f16, const void *q_bf16, void *q_f16, int64_t q_values, void *stream);
+                     void *v_f16, const void *q_bf16, void *q_f16, int64_t q_values, void *stream, bool pdl);
 bool decode_fp8_supported(int d_qk, int d_v, int hkv, int group, int block_size);
 int launch_decode_mma(const AttnParams &p, void *stream);
 int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas, bool alone);

@@ -264,102 +264,113 @@ __global__ void __launch_bounds__(kThreads, 2) prefill_fp8_kernel(const AttnPara
     }
 }
 
-// One staged block (a CTA): the 16 slots x 4 heads x 128 columns of K and of
-// V of a source block, dequantised (code value x row scale, rounded to f16)
+// One kv head of a staged block (a CTA): its 16 slots x 128 columns of K and of V
+// of a source block, dequantised (code value x row scale, rounded to f16)
 // into the plain cache layout [slot][head][column]; slots past `valid` are
 // zero. K rows: a thread writes 16 columns from the four words that hold them
 // (column 16 k + j at byte 32 c + 4 k + r); V: a thread reads one stored
 // column (16 slots, 16 bytes; a warp reads 512 contiguous bytes) and writes
 // its 16 values into their rows (a warp writes 64 contiguous bytes a row).
-__device__ __forceinline__ void fp8_dequant_block(const uint8_t *__restrict__ kp, const uint8_t *__restrict__ vp,
-                                                  const Fp8StageJob jb, uint4 *__restrict__ kd,
-                                                  uint4 *__restrict__ vd) {
+__device__ __forceinline__ void fp8_dequant_head(const uint8_t *__restrict__ kp, const uint8_t *__restrict__ vp,
+                                                 const Fp8StageJob jb, int head, uint4 *__restrict__ kd,
+                                                 uint4 *__restrict__ vd) {
     const uint8_t *kb = kp + static_cast<int64_t>(jb.src) * kBlockBytes;
     const uint8_t *vb = vp + static_cast<int64_t>(jb.src) * kBlockBytes;
-    const float *ksc = reinterpret_cast<const float *>(kb + kCodeBytes);
-    const float *vsc = reinterpret_cast<const float *>(vb + kCodeBytes);
-    uint4 *ko = kd + static_cast<int64_t>(jb.dst) * (kBs * kHkv * kD / 8);
-    uint4 *vo = vd + static_cast<int64_t>(jb.dst) * (kBs * kHkv * kD / 8);
+    const float *ksc = reinterpret_cast<const float *>(kb + kCodeBytes) + head;
+    const float *vsc = reinterpret_cast<const float *>(vb + kCodeBytes) + head;
+    const int slot = threadIdx.x >> 3, cg = threadIdx.x & 7;  // K: slot x 16 columns
+    const int d = threadIdx.x;                                // V: column
+    const int row = slot * kHkv + head;
+    uint32_t kw[4];  // every load in flight before the first use
+#pragma unroll
+    for (int c = 0; c < 4; ++c) kw[c] = __ldg(reinterpret_cast<const uint32_t *>(kb + row * kD + 32 * c + 4 * cg));
+    const uint4 w = __ldg(reinterpret_cast<const uint4 *>(vb + head * (kD * kBs) + d * kBs));
+    const float ks = __ldg(ksc + slot * kHkv);
+    float vs[kBs];
+#pragma unroll
+    for (int o = 0; o < kBs; ++o) vs[o] = __ldg(vsc + o * kHkv);
     auto scaled = [](uint32_t h2, float sc) {  // f16x2 * sc, rounded to f16x2
         const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&h2));
         return pack_f16x2(f.x * sc, f.y * sc);
     };
-    for (int task = threadIdx.x; task < kBs * kHkv * 8; task += 128) {  // K: row (slot, head) x 16 columns
-        const int row = task >> 3, cg = task & 7;
-        uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-        if ((row >> 2) < jb.valid) {
-            const float sc = ksc[row];
-            uint32_t lo[4], hi[4];
+    uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+    if (slot < jb.valid) {
+        uint32_t lo[4], hi[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                e4m3x4_to_f16x2x2(__ldg(reinterpret_cast<const uint32_t *>(kb + row * kD + 32 * c + 4 * cg)), lo[c], hi[c]);
-                lo[c] = scaled(lo[c], sc);
-                hi[c] = scaled(hi[c], sc);
-            }
-            a = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-            b = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        for (int c = 0; c < 4; ++c) {
+            e4m3x4_to_f16x2x2(kw[c], lo[c], hi[c]);
+            lo[c] = scaled(lo[c], ks);
+            hi[c] = scaled(hi[c], ks);
         }
-        ko[row * (kD / 8) + 2 * cg] = a;
-        ko[row * (kD / 8) + 2 * cg + 1] = b;
+        a = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        b = make_uint4(hi[0], hi[1], hi[2], hi[3]);
     }
-    __half *vh = reinterpret_cast<__half *>(vo);
-    for (int task = threadIdx.x; task < kHkv * kD; task += 128) {  // V: one stored column (head, d), 16 slots
-        const int head = task >> 7, d = task & (kD - 1);
-        const uint4 w = __ldg(reinterpret_cast<const uint4 *>(vb + head * (kD * kBs) + d * kBs));
-        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+    uint4 *ko = kd + static_cast<int64_t>(jb.dst) * (kBs * kHkv * kD / 8) + row * (kD / 8) + 2 * cg;
+    ko[0] = a;
+    ko[1] = b;
+    __half *vh = reinterpret_cast<__half *>(vd + static_cast<int64_t>(jb.dst) * (kBs * kHkv * kD / 8)) + head * kD + d;
+    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {  // word c: slots 2c, 2c + 1 (lo) and 2c + 8, 2c + 9 (hi)
-            uint32_t lo, hi;
-            e4m3x4_to_f16x2x2(ws[c], lo, hi);
-            const float2 fl = __half22float2(*reinterpret_cast<const __half2 *>(&lo));
-            const float2 fh = __half22float2(*reinterpret_cast<const __half2 *>(&hi));
-            const int sl[4] = {2 * c, 2 * c + 1, 2 * c + 8, 2 * c + 9};
-            const float f[4] = {fl.x, fl.y, fh.x, fh.y};
+    for (int c = 0; c < 4; ++c) {  // word c: slots 2c, 2c + 1 (lo) and 2c + 8, 2c + 9 (hi)
+        uint32_t lo, hi;
+        e4m3x4_to_f16x2x2(ws[c], lo, hi);
+        const float2 fl = __half22float2(*reinterpret_cast<const __half2 *>(&lo));
+        const float2 fh = __half22float2(*reinterpret_cast<const __half2 *>(&hi));
+        const int sl[4] = {2 * c, 2 * c + 1, 2 * c + 8, 2 * c + 9};
+        const float f[4] = {fl.x, fl.y, fh.x, fh.y};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int o = sl[e];
-                vh[(o * kHkv + head) * kD + d] =
-                    __float2half_rn(o < jb.valid ? f[e] * vsc[o * kHkv + head] : 0.f);
-            }
-        }
+        for (int e = 0; e < 4; ++e)
+            vh[sl[e] * (kHkv * kD)] = __float2half_rn(sl[e] < jb.valid ? f[e] * vs[sl[e]] : 0.f);
     }
 }
 
-// The staging in one launch: CTAs below num_jobs dequantise one block each,
-// the others convert the queries bf16 -> f16 (8 values per thread and step).
+// The staging in one launch: CTAs below 4 num_jobs dequantise one kv head of
+// one block each, the others convert the queries bf16 -> f16, 8 values per load
+// and kQUnroll loads in flight a thread. Latency-bound: 128 blocks and 2176
+// tokens of 28 heads took 12.5 us with one CTA per block, its loads one after
+// another, and one load in flight a thread; 10.4 us so (34 MB, from a cold L2).
+constexpr int kQUnroll = 4;
 __global__ void __launch_bounds__(128) fp8_stage_kernel(const uint8_t *__restrict__ kp, const uint8_t *__restrict__ vp,
                                                         const Fp8StageJob *__restrict__ jobs, int32_t num_jobs,
                                                         uint4 *__restrict__ kd, uint4 *__restrict__ vd,
                                                         const uint4 *__restrict__ qin, uint4 *__restrict__ qout,
                                                         int64_t n8) {
-    if (static_cast<int32_t>(blockIdx.x) < num_jobs) {
-        fp8_dequant_block(kp, vp, jobs[blockIdx.x], kd, vd);
+    pdl_trigger();
+    pdl_wait();  // the codes of the kernel before (the step's append)
+    if (static_cast<int32_t>(blockIdx.x) < kHkv * num_jobs) {
+        fp8_dequant_head(kp, vp, jobs[blockIdx.x / kHkv], blockIdx.x % kHkv, kd, vd);
         return;
     }
-    const int64_t nq = static_cast<int64_t>(gridDim.x) - num_jobs;
-    for (int64_t i = (static_cast<int64_t>(blockIdx.x) - num_jobs) * blockDim.x + threadIdx.x; i < n8;
-         i += nq * blockDim.x) {
-        const uint4 v = __ldg(qin + i);
-        qout[i] = make_uint4(bf16x2_to_f16x2(v.x), bf16x2_to_f16x2(v.y), bf16x2_to_f16x2(v.z), bf16x2_to_f16x2(v.w));
+    const int64_t nq = static_cast<int64_t>(gridDim.x) - kHkv * num_jobs;
+    for (int64_t i = (static_cast<int64_t>(blockIdx.x) - kHkv * num_jobs) * (kQUnroll * 128) + threadIdx.x; i < n8;
+         i += nq * (kQUnroll * 128)) {
+        uint4 v[kQUnroll];
+#pragma unroll
+        for (int u = 0; u < kQUnroll; ++u) v[u] = i + 128 * u < n8 ? __ldg(qin + i + 128 * u) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < kQUnroll; ++u)
+            if (i + 128 * u < n8)
+                qout[i + 128 * u] = make_uint4(bf16x2_to_f16x2(v[u].x), bf16x2_to_f16x2(v[u].y), bf16x2_to_f16x2(v[u].z),
+                                               bf16x2_to_f16x2(v[u].w));
     }
 }
 
 }  // namespace
 
 int launch_fp8_stage(const void *k_pool, const void *v_pool, const Fp8StageJob *jobs, int32_t num_jobs, void *k_f16,
-                     void *v_f16, const void *q_bf16, void *q_f16, int64_t q_values, void *stream) {
+                     void *v_f16, const void *q_bf16, void *q_f16, int64_t q_values, void *stream, bool pdl) {
     const int64_t n8 = q_values / 8;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t want = (n8 + 127) / 128;
-    const int64_t qctas = want < 4LL * sms ? want : 4LL * sms;
+    const int64_t want = (n8 + kQUnroll * 128 - 1) / (kQUnroll * 128);
+    const int64_t qctas = want < 16LL * sms ? want : 16LL * sms;  // (one wave at most: 16 CTAs a SM)
     if (num_jobs + qctas == 0) return FNPU_OK;
-    fp8_stage_kernel<<<static_cast<int>(num_jobs + qctas), 128, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint8_t *>(k_pool), static_cast<const uint8_t *>(v_pool), jobs, num_jobs,
-        static_cast<uint4 *>(k_f16), static_cast<uint4 *>(v_f16), static_cast<const uint4 *>(q_bf16),
-        static_cast<uint4 *>(q_f16), n8);
-    FNPU_CUDA_TRY(cudaGetLastError());
+    FNPU_CUDA_TRY(launch_ex(fp8_stage_kernel, static_cast<int>(kHkv * num_jobs + qctas), 128, 0,
+                            static_cast<cudaStream_t>(stream), pdl, nullptr, static_cast<const uint8_t *>(k_pool),
+                            static_cast<const uint8_t *>(v_pool), jobs, num_jobs, static_cast<uint4 *>(k_f16),
+                            static_cast<uint4 *>(v_f16), static_cast<const uint4 *>(q_bf16),
+                            static_cast<uint4 *>(q_f16), n8));
     return FNPU_OK;
 }
 

@@ -126,6 +126,41 @@ def test_fp8_append_skips_padding_and_flags_out_of_range():
     assert np.array_equal(before[0], after[0]) and np.array_equal(before[1], after[1])
 
 
+@pytest.mark.parametrize("order", ["aligned", "offset", "nine", "ten", "reversed", "swapped", "holes", "two runs", "long"])
+def test_fp8_append_whole_words_and_single_rows_agree(order):
+    """The V rows of slots 2 c, 2 c + 1, 2 c + 8, 2 c + 9 of a block are stored as
+    words when one call brings the four in slot order, else byte by byte, and a
+    call of more than one wave ("long") has a token's K rows in one warp: any
+    order of slots leaves the same bytes as one call per token, in the first and
+    the last block of the pool as well."""
+    import paper_2606_04415_gb300 as fnpu
+    from paper_2606_04415_gb300.step import DeviceStep
+    batch = _batch([1000], seed=4)
+    n = batch.num_blocks * 16
+    up = lambda b, e: list(range(b, e))
+    slots = {
+        "aligned": up(0, 48), "offset": up(5, 61), "nine": up(16, 25), "ten": up(16, 26),
+        "reversed": up(0, 32)[::-1], "swapped": up(0, 8) + up(9, 10) + up(8, 9) + up(10, 32),
+        "holes": up(0, 5) + [-1] + up(6, 24) + [-1, -1] + up(26, 40),
+        "long": up(7, 7 + 5 * torch.cuda.get_device_properties(0).multi_processor_count + 1),
+        "two runs": up(n - 20, n) + up(3, 35)}[order]
+    T = len(slots)
+    rng = np.random.default_rng(7)
+    bits = W.f32_to_bf16_bits(rng.standard_normal((2, T, 4, 128)).astype(np.float32))
+    rows = torch.from_numpy(bits.view(np.int16)).cuda().view(torch.bfloat16)
+    sl = torch.tensor(slots, dtype=torch.int64, device="cuda")
+    init = W.stale_pool_bytes(batch.num_blocks * F8.block_bytes(4), 4)
+    pools = []
+    for step in (T, 1):
+        st = DeviceStep(batch, kv_fp8=True, pool_init=init)
+        for t in range(0, T, step):
+            fnpu.kv_append(st.desc, rows[0, t:t + step], rows[1, t:t + step], sl[t:t + step], st.k_cache, st.v_cache)
+        assert fnpu.check() == fnpu.FNPU_OK
+        pools.append(st.cache_bits())
+    assert np.array_equal(pools[0][0], pools[1][0])
+    assert np.array_equal(pools[0][1], pools[1][1])
+
+
 @pytest.mark.parametrize("hq", [4, 16, 28, 32])
 @pytest.mark.parametrize("split", [0, 64, 192])
 def test_fp8_decode_ragged_groups_and_splits(hq, split):
