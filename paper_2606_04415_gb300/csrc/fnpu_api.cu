@@ -179,70 +179,8 @@ void release_plan(fnpu_plan *pl) {
 // whole device about 4 TB/s.
 constexpr double kTileSec = 1.5e-6;
 constexpr double kDecodeSmBps = 69e9;
+constexpr double kDecodeSmBpsFp8 = 50e9;  // (bytes of the FP8 cache: the conversion bounds it)
 constexpr double kDecodeAllBps = 4.0e12;
-
-// (stop_at: the run may end as soon as the makespan reaches it; loads, if
-// given, receives the final number of workers per load)
-int64_t lpt_makespan(const std::vector<int32_t> &hist, int32_t m, int64_t stop_at = INT64_MAX,
-                     std::vector<int32_t> *loads = nullptr);
-std::vector<int32_t> cost_histogram(const std::vector<int64_t> &costs);
-
-// SMs that start on decode while the others run prefill: the prefill CTAs on
-// sms - k SMs take the items longest first, so each ends at its load of the
-// LPT schedule of the item costs on sms - k workers, the last at the makespan
-// Tp. Decode streams at min(all, per SM x SMs it holds) on the k SMs from the
-// start and on each prefill SM from the moment its CTA ends (its CTAs take
-// the SMs the prefill leaves), until the decode bytes are read at Td. The k
-// with the shortest modelled step max(Tp, Td) wins, the largest such k on
-// ties (more decode done while the prefill lasts).
-int32_t choose_decode_sms(const std::vector<int64_t> &item_tiles, double tile_scale, int64_t dec_bytes,
-                          int32_t sms) {
-    const std::vector<int32_t> hist = cost_histogram(item_tiles);
-    const double unit = tile_scale * kTileSec;  // seconds per cost unit
-    std::vector<int32_t> loads;
-    // (prefill end, decode end) with k decode SMs
-    auto phases = [&](int32_t k) {
-        const double tp = static_cast<double>(lpt_makespan(hist, sms - k, INT64_MAX, &loads)) * unit;
-        double left = static_cast<double>(dec_bytes), t = 0.0;
-        int32_t n = k;
-        for (size_t ld = 0; ld <= loads.size() && left > 0.0; ++ld) {
-            // decode on n SMs until the next prefill CTAs end (at load ld)
-            const double next = ld < loads.size() ? static_cast<double>(ld) * unit : 1e30;
-            if (ld < loads.size() && loads[ld] == 0) continue;
-            const double rate = std::min(kDecodeAllBps, n * kDecodeSmBps);
-            if (next > t) {
-                const double run = std::min(next - t, left / rate);
-                left -= run * rate;
-                t += run;
-            }
-            if (ld < loads.size()) n += loads[ld];
-        }
-        return std::make_pair(tp, t);
-    };
-    // The prefill end grows with k and the decode end shrinks, so the step
-    // max(Tp, Td) is shortest near the smallest k whose decode ends within
-    // the prefill: found by bisection, then the k around it are compared
-    // (the LPT makespan is not strictly monotone in the number of workers)
-    const int32_t kmax = std::max<int32_t>(sms / 2, 1);
-    int32_t lo = 1, hi = kmax;
-    while (lo < hi) {
-        const int32_t mid = (lo + hi) / 2;
-        const auto ph = phases(mid);
-        if (ph.second <= ph.first) hi = mid;
-        else lo = mid + 1;
-    }
-    int32_t best_k = 1;
-    double best_t = -1.0;
-    for (int32_t k = std::max<int32_t>(1, lo - 4); k <= std::min<int32_t>(kmax, lo + 4); ++k) {
-        const auto ph = phases(k);
-        const double step = std::max(ph.first, ph.second);
-        if (best_t < 0 || step <= best_t) {
-            best_t = step;
-            best_k = k;
-        }
-    }
-    return best_k;
-}
 
 // Two packed Q tiles of one kv head (the tcgen05 prefill unit) before its key
 // range is split.
@@ -269,6 +207,105 @@ constexpr int32_t kDualTiles = 4;
 // First tile of split j of n over ntiles tiles (split n is the end).
 int32_t split_bound(int32_t ntiles, int32_t n, int32_t j) {
     return static_cast<int32_t>((static_cast<int64_t>(ntiles) * j) / n);
+}
+
+// Pieces that the remainder of the units may be cut into (see wave_units).
+constexpr int32_t kMaxRemainderPieces = 4;
+
+// Units by decreasing length, the candidates for a schedule that takes whole
+// waves of them as they are and cuts only the remainder, the U mod m shortest
+// ones, into n pieces each. (Cut at a cap, every unit longer than it pays the
+// partial write and the merge; a remainder of a few units costs a wave of its
+// own if nothing is cut.)
+struct WaveUnits {
+    std::vector<int32_t> order;   // unit indices, longest first
+    std::vector<int32_t> ntiles;  // their lengths
+    std::vector<int32_t> nmax;    // pieces they can take, at most kMaxRemainderPieces
+};
+// (empty if a unit has one Q tile: those have caps of their own)
+WaveUnits wave_units(const std::vector<TcUnit> &units);
+// Histogram of the item costs with the remainder on m workers in n pieces;
+// false if there is no remainder, less than a wave, or a unit that cannot be cut so.
+bool remainder_histogram(const WaveUnits &w, int32_t m, int32_t n, std::vector<int32_t> *hist);
+
+// (stop_at: the run may end as soon as the makespan reaches it; loads, if
+// given, receives the final number of workers per load)
+int64_t lpt_makespan(const std::vector<int32_t> &hist, int32_t m, int64_t stop_at = INT64_MAX,
+                     std::vector<int32_t> *loads = nullptr);
+std::vector<int32_t> cost_histogram(const std::vector<int64_t> &costs);
+
+// SMs that start on decode while the others run prefill: the prefill CTAs on
+// sms - k SMs take the items longest first, so each ends at its load of the
+// LPT schedule of the item costs on sms - k workers, the last at the makespan
+// Tp. Decode streams at min(all, per SM x SMs it holds) on the k SMs from the
+// start and on each prefill SM from the moment its CTA ends (its CTAs take
+// the SMs the prefill leaves), until the decode bytes are read at Td. The k
+// with the shortest modelled step max(Tp, Td) wins, the largest such k on
+// ties (more decode done while the prefill lasts).
+// `wave`, if not null: with the remainder of the units in pieces, for k near the
+// choice without (host time: each k is some schedules).
+struct DecodeShare {
+    int32_t k;
+    double step;  // modelled seconds
+};
+DecodeShare choose_decode_sms(const std::vector<int64_t> &item_tiles, const WaveUnits *wave, double tile_scale,
+                              int64_t dec_bytes, double sm_bps, int32_t sms, int32_t near = 1) {
+    const std::vector<int32_t> hist = cost_histogram(item_tiles);
+    const double unit = tile_scale * kTileSec;  // seconds per cost unit
+    std::vector<int32_t> loads, rloads, rh;
+    // (prefill end, decode end) with k decode SMs
+    auto phases = [&](int32_t k) {
+        int64_t span = INT64_MAX;
+        for (int32_t n = 2; wave && n <= kMaxRemainderPieces; ++n) {
+            if (!remainder_histogram(*wave, sms - k, n, &rh)) break;
+            const int64_t rs = lpt_makespan(rh, sms - k, span, &rloads);
+            if (rs >= span) break;
+            span = rs;
+            loads.swap(rloads);
+        }
+        if (span == INT64_MAX) span = lpt_makespan(hist, sms - k, INT64_MAX, &loads);
+        const double tp = static_cast<double>(span) * unit;
+        double left = static_cast<double>(dec_bytes), t = 0.0;
+        int32_t n = k;
+        for (size_t ld = 0; ld <= loads.size() && left > 0.0; ++ld) {
+            // decode on n SMs until the next prefill CTAs end (at load ld)
+            const double next = ld < loads.size() ? static_cast<double>(ld) * unit : 1e30;
+            if (ld < loads.size() && loads[ld] == 0) continue;
+            const double rate = std::min(kDecodeAllBps, n * sm_bps);
+            if (next > t) {
+                const double run = std::min(next - t, left / rate);
+                left -= run * rate;
+                t += run;
+            }
+            if (ld < loads.size()) n += loads[ld];
+        }
+        return std::make_pair(tp, t);
+    };
+    // The prefill end grows with k and the decode end shrinks, so the step
+    // max(Tp, Td) is shortest near the smallest k whose decode ends within
+    // the prefill: found by bisection, then the k around it are compared
+    // (the LPT makespan is not strictly monotone in the number of workers)
+    const int32_t kmax = std::max<int32_t>(sms / 2, 1);
+    int32_t lo = wave ? std::max<int32_t>(1, near - 2) : 1;
+    int32_t hi = wave ? std::min<int32_t>(kmax, 2 * near + 16) : kmax;
+    const int32_t around = wave ? 2 : 4;
+    while (lo < hi) {
+        const int32_t mid = (lo + hi) / 2;
+        const auto ph = phases(mid);
+        if (ph.second <= ph.first) hi = mid;
+        else lo = mid + 1;
+    }
+    int32_t best_k = 1;
+    double best_t = -1.0;
+    for (int32_t k = std::max<int32_t>(1, lo - around); k <= std::min<int32_t>(kmax, lo + around); ++k) {
+        const auto ph = phases(k);
+        const double step = std::max(ph.first, ph.second);
+        if (best_t < 0 || step <= best_t) {
+            best_t = step;
+            best_k = k;
+        }
+    }
+    return DecodeShare{best_k, best_t};
 }
 
 // Item costs (positive integers, in tiles) as a histogram: hist[c] items of
@@ -344,12 +381,47 @@ std::vector<int32_t> longest_first(const std::vector<int64_t> &cost) {
     return order;
 }
 
+WaveUnits wave_units(const std::vector<TcUnit> &units) {
+    WaveUnits w;
+    for (const TcUnit &u : units)
+        if (u.dual) return w;
+    std::vector<int64_t> cost(units.size());
+    for (size_t i = 0; i < units.size(); ++i) cost[i] = units[i].ntiles;
+    w.order = longest_first(cost);
+    w.ntiles.reserve(units.size());
+    w.nmax.reserve(units.size());
+    for (int32_t i : w.order) {
+        w.ntiles.push_back(units[i].ntiles);
+        int32_t n = std::min<int32_t>(kMaxRemainderPieces, std::max<int32_t>(units[i].ntiles, 1));
+        while (n > 1 && split_bound(units[i].ntiles, n, n - 1) > units[i].max_start) --n;
+        w.nmax.push_back(n);
+    }
+    return w;
+}
+
+bool remainder_histogram(const WaveUnits &w, int32_t m, int32_t n, std::vector<int32_t> *out) {
+    const size_t nu = w.order.size();
+    if (m < 1 || nu <= static_cast<size_t>(m) || nu % static_cast<size_t>(m) == 0) return false;
+    const size_t first = nu - nu % static_cast<size_t>(m);  // of the remainder
+    for (size_t i = first; i < nu; ++i)
+        if (w.nmax[i] < n) return false;
+    std::vector<int32_t> &hist = *out;
+    hist.assign(static_cast<size_t>(w.ntiles[0] + kTcItemCost + kTcMergeCost) + 1, 0);
+    for (size_t i = 0; i < first; ++i) ++hist[static_cast<size_t>(w.ntiles[i] + kTcItemCost)];
+    for (size_t i = first; i < nu; ++i) {  // (as in split_bound: the longer pieces are ntiles mod n of them)
+        const int32_t q = w.ntiles[i] / n, r = w.ntiles[i] % n;
+        hist[static_cast<size_t>(q + 1 + kTcItemCost + kTcMergeCost)] += r;
+        hist[static_cast<size_t>(q + kTcItemCost + kTcMergeCost)] += n - r;
+    }
+    return true;
+}
+
 // Number of key splits per unit. A persistent CTA per SM takes items longest
 // first, so the step lasts about as long as the LPT schedule of the items.
 // Splitting the largest units evens that schedule out but costs a partial
 // write and a merge, so the piece-size cap is chosen among a few candidates
 // by the modelled makespan.
-std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, int32_t sms) {
+std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, bool cut, int32_t sms) {
     int64_t total = 0, maxc = 0;
     for (const TcUnit &u : units) {
         total += u.ntiles;
@@ -446,6 +518,21 @@ std::vector<int32_t> choose_prefill_splits(const std::vector<TcUnit> &units, int
         if (best_span < 0 || span < best_span) {
             best_span = span;
             best = ns;
+        }
+    }
+    // the remainder of the last wave in pieces, where a ninth could be gained
+    // (2048 tokens of 28 heads on 6000 keys, 228 units: 157 us a step with every
+    // unit cut in two, 141 so; 1600 on 3000, 180 units: 86.8 whole, 78)
+    cut = cut && static_cast<int32_t>(units.size()) > sms && 9 * ((whole + sms - 1) / sms) <= 8 * best_span;
+    WaveUnits wave;
+    if (cut) wave = wave_units(units);
+    for (int32_t n = 2; cut && n <= kMaxRemainderPieces; ++n) {
+        if (!remainder_histogram(wave, sms, n, &hist)) break;
+        const int64_t span = lpt_makespan(hist, sms, best_span);
+        if (span < best_span) {
+            best_span = span;
+            std::fill(best.begin(), best.end(), 1);
+            for (size_t i = units.size() - units.size() % static_cast<size_t>(sms); i < units.size(); ++i) best[wave.order[i]] = n;
         }
     }
     return best;
@@ -913,6 +1000,7 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
         for (const TcUnit &u : tc_units) longest = std::max(longest, u.ntiles);
         pl->coloc = static_cast<double>(longest + kTcItemCost) * tile_scale * kTileSec >= 5e-6;
     }
+    bool cut = !pl->coloc;  // to cut the remainder of the last wave of units, where there is one
     pl->pre_ctas = sms;
     if (pl->coloc) {
         int64_t dec_bytes = 0;
@@ -923,9 +1011,32 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
         std::vector<int64_t> item_tiles;
         for (const TcUnit &u : tc_units) item_tiles.push_back(u.ntiles + kTcItemCost);
         std::sort(item_tiles.begin(), item_tiles.end(), [](int64_t a, int64_t b) { return a > b; });
-        const int32_t k = o.decode_share_pct > 0
-                              ? std::min(sms - 1, std::max(1, (sms * o.decode_share_pct + 50) / 100))
-                              : choose_decode_sms(item_tiles, tile_scale, dec_bytes, sms);
+        int32_t k;
+        if (o.decode_share_pct > 0) {
+            k = std::min(sms - 1, std::max(1, (sms * o.decode_share_pct + 50) / 100));
+        } else {
+            // Whole units leave SMs to the decode as their last wave runs out;
+            // cutting that wave's remainder (see wave_units) takes them back and
+            // adds the merges. It is done only where the model has the step a
+            // ninth shorter: 81 -> 70.5 us by the model (1024 tokens on 3000 and
+            // 64 decodes, 8 kv heads) measured 97.5 -> 91, 93 -> 67.5 (FP8 cache)
+            // 112 -> 99, 111 -> 97.5 125 -> 113.5; but 60 -> 54 measured 79.6 -> 83.5
+            // and 85.5 -> 81 97 -> 100. (No schedule is shorter than the work
+            // of both phases over all SMs, which rules most steps out.)
+            const double sm_bps = desc->kv_fp8 ? kDecodeSmBpsFp8 : kDecodeSmBps;
+            const DecodeShare whole = choose_decode_sms(item_tiles, nullptr, tile_scale, dec_bytes, sm_bps, sms);
+            k = whole.k;
+            int64_t work = 0;
+            for (int64_t t : item_tiles) work += t;
+            const double least = (static_cast<double>(work) * tile_scale * kTileSec + dec_bytes / sm_bps) / sms;
+            if (9 * least <= 8 * whole.step && static_cast<int32_t>(tc_units.size()) > sms - whole.k) {
+                const WaveUnits wave = wave_units(tc_units);
+                const DecodeShare pieces =
+                    choose_decode_sms(item_tiles, &wave, tile_scale, dec_bytes, sm_bps, sms, whole.k);
+                cut = 9 * pieces.step <= 8 * whole.step;
+                if (cut) k = pieces.k;
+            }
+        }
         pl->pre_ctas = sms - k;
         if ((o.flags & FNPU_PLAN_GREEN_CONTEXTS) && pl->g_pre && pl->green_k == k) {
             pl->pre_ctas = pl->green_pre;  // the partitions of the last plan fit this share
@@ -968,7 +1079,7 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
     int32_t pparts = 0, pgroups = 0;
     pl->pitems_dual = 0;
     if (!tc_units.empty()) {
-        const std::vector<int32_t> ns = choose_prefill_splits(tc_units, pl->pre_ctas);
+        const std::vector<int32_t> ns = choose_prefill_splits(tc_units, cut, pl->pre_ctas);
         for (size_t u = 0; u < tc_units.size(); ++u) {
             const TcUnit &t = tc_units[u];
             const int32_t n = ns[u];

@@ -326,6 +326,25 @@ def test_single_q_tile_items(heads, dim, bs):
         assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
 
 
+@pytest.mark.parametrize("prefix,decodes,cut", [(2000, 0, True), (2000, 6, None), (63, 0, False)])
+def test_remainder_of_the_last_wave_in_pieces(prefix, decodes, cut):
+    """14 tile pairs on 12 SMs: the two that do not fit one wave are cut into
+    pieces of their keys and merged, the others stay whole (a short prefix, whose
+    rows do not all see every piece, is left whole), alone and beside decodes."""
+    sh = W.Shape(8, 2, 128, 128, 32, False)
+    ql, ctx, ph = [448] + [1] * decodes, [448 + prefix] + [300 + 217 * i for i in range(decodes)], [0] + [1] * decodes
+    batch = W.build_batch(sh, ql, ctx, ph, np.random.default_rng(prefix + decodes), name="remainder")
+    st = _step(batch, sms=12)
+    items = st.plan.info()["prefill_items"]
+    if cut is not None:
+        assert (14 < items <= 12 + 2 * 4) if cut else items == 14
+    out, lse = st.results()
+    _compare(batch, out, lse, tokens=_sample_tokens(batch, per_seq_rows=24))
+    st.run()
+    out2, lse2 = st.results()
+    assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
+
+
 SEPARATE = 1  # FNPU_PLAN_SEPARATE_LAUNCHES
 
 
