@@ -988,29 +988,33 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
     pl->coloc = pl->use_tc && pl->use_dt && !tc_units.empty() && !ditems.empty() &&
                 !(o.flags & FNPU_PLAN_SEPARATE_LAUNCHES);
     const double tile_scale = (desc->head_dim_qk + desc->head_dim_v) / 256.0;  // relative to d = 128
-    if (pl->coloc && desc->num_kv_heads != 4 && o.decode_share_pct == 0 && !(o.flags & FNPU_PLAN_GREEN_CONTEXTS)) {
-        // A prefill of one or two short tiles is over before the fork, the
-        // join and the wait for its start are paid for: with a chunk of 128
-        // tokens, d = 64 and no prefix (2.3 us by the model) a re-planned
-        // step takes 28.6 us with the phases in turn and 42.6 co-located;
-        // from about 5 us on co-location wins (chunks of 32 to 512 tokens:
-        // 26.6 us against 28.7, 32.9 against 39.6, 35.6 against 43.1). Four kv
-        // heads co-locate always: such plans report phase times.
-        int32_t longest = 0;
-        for (const TcUnit &u : tc_units) longest = std::max(longest, u.ntiles);
-        pl->coloc = static_cast<double>(longest + kTcItemCost) * tile_scale * kTileSec >= 5e-6;
-    }
-    bool cut = !pl->coloc;  // to cut the remainder of the last wave of units, where there is one
-    pl->pre_ctas = sms;
+    std::vector<int64_t> item_tiles;
+    int64_t dec_bytes = 0;
     if (pl->coloc) {
-        int64_t dec_bytes = 0;
+        for (const TcUnit &u : tc_units) item_tiles.push_back(u.ntiles + kTcItemCost);
         for (const DecodeItem &it : ditems)
             dec_bytes += static_cast<int64_t>(it.key_end - it.key_begin) * std::min(hpi, desc->num_kv_heads - it.kvh) *
                          (desc->kv_fp8 ? desc->head_dim_qk + desc->head_dim_v + 8
                                        : (desc->head_dim_qk + desc->head_dim_v) * 2);
-        std::vector<int64_t> item_tiles;
-        for (const TcUnit &u : tc_units) item_tiles.push_back(u.ntiles + kTcItemCost);
-        std::sort(item_tiles.begin(), item_tiles.end(), [](int64_t a, int64_t b) { return a > b; });
+    }
+    if (pl->coloc && desc->num_kv_heads != 4 && o.decode_share_pct == 0 && !(o.flags & FNPU_PLAN_GREEN_CONTEXTS)) {
+        // The fork, the wait for the prefill's start and the join cost a step
+        // some 5 us; what co-location saves is the decode's time. It is worth
+        // it for a long decode (20 us by the model, 80 MB: 111 of 100 .. 3500
+        // keys beside 78 tokens on 1000, 94 us a step in turn, 84.5 together),
+        // or a prefill long enough to have a light one in its slack: of 8 us
+        // where its units leave SMs free (d = 64, 1080 tokens on 7 and 35
+        // decodes: 33.4, 29.5; below, 9.8 MB and 6 us: 23.9, 26.3), of 25 us
+        // where they do not (219 x 3 tokens on 5223: 78.9, 58.2; but 1603 tokens
+        // on 2 and 35 short decodes, 22.5 us by the model: 42.2, 47.5). Four kv
+        // heads co-locate always: such plans report phase times.
+        const double span = static_cast<double>(lpt_makespan(cost_histogram(item_tiles), sms)) * tile_scale * kTileSec;
+        const bool wide = 4 * static_cast<int64_t>(tc_units.size()) > 3 * static_cast<int64_t>(sms);
+        pl->coloc = span >= (dec_bytes >= 20e-6 * kDecodeAllBps ? 5e-6 : wide ? 25e-6 : 8e-6);
+    }
+    bool cut = !pl->coloc;  // to cut the remainder of the last wave of units, where there is one
+    pl->pre_ctas = sms;
+    if (pl->coloc) {
         int32_t k;
         if (o.decode_share_pct > 0) {
             k = std::min(sms - 1, std::max(1, (sms * o.decode_share_pct + 50) / 100));

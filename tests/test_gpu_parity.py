@@ -345,6 +345,24 @@ def test_remainder_of_the_last_wave_in_pieces(prefix, decodes, cut):
     assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
 
 
+@pytest.mark.parametrize("prefix,sms,together", [(40, 16, False), (1500, 16, True), (1500, 8, False), (6000, 8, True)])
+def test_light_decode_beside_or_after_the_prefill(prefix, sms, together):
+    """Eight kv heads, so eight tile pairs: a light decode runs beside a prefill
+    that is long enough, which is sooner so where SMs stay free (8 pairs on 16)
+    than where they do not (8 on 8), and otherwise after it."""
+    import paper_2606_04415_gb300 as fnpu
+    sh = W.Shape(16, 8, 64, 64, 16, False)
+    batch = W.build_batch(sh, [100, 1, 1, 1], [100 + prefix, 30, 311, 900], [0, 1, 1, 1], np.random.default_rng(prefix + sms),
+                          name="light_decode")
+    st = _step(batch, sms=sms)
+    if together:
+        fnpu.plan_phase_ms(st.plan)
+    else:
+        with pytest.raises(fnpu.FnpuError):
+            fnpu.plan_phase_ms(st.plan)
+    _compare(batch, *st.results(), tokens=_sample_tokens(batch, per_seq_rows=24))
+
+
 SEPARATE = 1  # FNPU_PLAN_SEPARATE_LAUNCHES
 
 
