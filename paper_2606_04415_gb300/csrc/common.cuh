@@ -119,7 +119,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\
 // `cooperative` (launch_coop) guarantees that every CTA of the grid is
 // resident at once, which a grid whose CTAs wait for one another needs.
 template <typename... Args>
-cudaError_t launch_coop(void (*kernel)(Args...), int grid, int threads, size_t smem, cudaStream_t st,
+cudaError_t launch_coop(void (*kernel)(Args...), dim3 grid, int threads, size_t smem, cudaStream_t st,
                         bool after_prev, cudaEvent_t started, bool cooperative, const Args &...args) {
     cudaLaunchAttribute attr[3];
     int n = 0;
@@ -140,7 +140,7 @@ cudaError_t launch_coop(void (*kernel)(Args...), int grid, int threads, size_t s
         ++n;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -149,7 +149,7 @@ cudaError_t launch_coop(void (*kernel)(Args...), int grid, int threads, size_t s
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 template <typename... Args>
-cudaError_t launch_ex(void (*kernel)(Args...), int grid, int threads, size_t smem, cudaStream_t st, bool after_prev,
+cudaError_t launch_ex(void (*kernel)(Args...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool after_prev,
                       cudaEvent_t started, const Args &...args) {
     return launch_coop(kernel, grid, threads, smem, st, after_prev, started, false, args...);
 }

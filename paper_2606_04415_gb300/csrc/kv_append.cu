@@ -285,6 +285,8 @@ __global__ void __launch_bounds__(256) mla_gather_kernel(const uint4 *__restrict
                                                          const int64_t *__restrict__ slots, int32_t n,
                                                          int64_t num_slots, int32_t heads,
                                                          uint4 *__restrict__ ws, uint4 *__restrict__ k_out) {
+    pdl_trigger();  // as in kv_append_kernel
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t step = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
     for (int64_t i = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5; i < n; i += step) {
@@ -316,10 +318,10 @@ int launch_mla_gather(const void *latent, const int64_t *slots, int32_t n, int64
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t want = (static_cast<int64_t>(n) + 7) / 8;  // 8 rows (warps) per block
     const int grid = static_cast<int>(want < 16LL * sms ? want : 16LL * sms);
-    mla_gather_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint4 *>(latent), slots, n, num_slots, heads, static_cast<uint4 *>(ws),
-        static_cast<uint4 *>(k_out));
-    return cudaGetLastError() == cudaSuccess ? FNPU_OK : FNPU_ECUDA;
+    FNPU_CUDA_TRY(launch_ex(mla_gather_kernel, grid, 256, 0, static_cast<cudaStream_t>(stream), true, nullptr,
+                            static_cast<const uint4 *>(latent), slots, n, num_slots, heads, static_cast<uint4 *>(ws),
+                            static_cast<uint4 *>(k_out)));
+    return FNPU_OK;
 }
 
 int global_error_address(int **out) {

@@ -28,6 +28,13 @@
 //     accumulators back (one row per thread), round to bf16 (nearest-even)
 //     into swizzled boxes in shared memory, and TMA stores write the key and
 //     value rows.
+// The append, the gather, the GEMM and the attention after it are programmatic
+// dependent launches of one another (1024 rows of 128 heads, the four together:
+// 110.8 -> 106.3 us). One persistent CTA per SM with the row tile resident in
+// shared memory and only the weights streaming (256 KB an item instead of 384,
+// with or without multicast to a second CTA) took the same time: 64 KB in
+// flight cover less of the latency than these CTAs' 192, and stores add 14 us to
+// its 27.
 // Every mbarrier wait is bounded; a timeout raises bit 2 of the library-wide
 // device error flag (fnpu_check: FNPU_EDEVICE_TIMEOUT) and the CTA drains its
 // tensor-core work, frees its tensor memory and exits.
@@ -72,6 +79,7 @@ __global__ void __launch_bounds__(kGThreads, 2)
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int tid = threadIdx.x, warp = tid >> 5;
     const int row0 = blockIdx.x * kGRows, h = blockIdx.y;
+    pdl_trigger();  // the attention after it may set up as these CTAs end
     if ((s_base & 1023u) != 0) {  // the swizzled boxes need 1024-byte alignment
         if (tid == 0) atomicOr(err, 4);
         return;
@@ -109,6 +117,7 @@ __global__ void __launch_bounds__(kGThreads, 2)
             tc::prefetch_tmap(&maps.wk);
             tc::prefetch_tmap(&maps.wv);
         }
+        pdl_wait();  // the workspace (the gather), and earlier readers of the outputs
         for (int c = 0; c < kGChunks; ++c) {
             const int st = c % kGStages;
             if (c >= kGStages && !wait(EMPTY(st), ((c / kGStages) - 1) & 1)) break;
@@ -287,8 +296,8 @@ extern "C" int fnpu_mla_expand(const fnpu_attn_desc *desc, const void *latent_ca
         return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled (MLA expansion)");
     FNPU_CUDA_TRY(cudaFuncSetAttribute(mla_expand_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem));
     const dim3 grid((n + kGRows - 1) / kGRows, heads);
-    mla_expand_gemm_kernel<<<grid, kGThreads, kGSmem, static_cast<cudaStream_t>(stream)>>>(
-        maps, n, heads, static_cast<__nv_bfloat16 *>(k_out), static_cast<__nv_bfloat16 *>(v_out), err);
-    FNPU_CUDA_TRY(cudaGetLastError());
+    FNPU_CUDA_TRY(launch_ex(mla_expand_gemm_kernel, grid, kGThreads, kGSmem, static_cast<cudaStream_t>(stream), true,
+                            nullptr, maps, n, static_cast<int32_t>(heads), static_cast<__nv_bfloat16 *>(k_out),
+                            static_cast<__nv_bfloat16 *>(v_out), err));
     return FNPU_OK;
 }
