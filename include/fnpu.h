@@ -264,7 +264,8 @@ int fnpu_plan_info(const fnpu_plan *plan, int32_t *prefill_items, int32_t *decod
  * including the split merge (*decode_ms). Blocks until that run has ended.
  *   Errors: FNPU_EINVAL for NULL arguments or a plan that has not run yet;
  *   FNPU_EUNSUPPORTED for a plan that does not co-locate (one phase only,
- *   latent attention, or FNPU_PLAN_SEPARATE_LAUNCHES).
+ *   latent attention, FNPU_PLAN_SEPARATE_LAUNCHES, or a number of kv heads
+ *   other than four and a step that is faster with its phases in turn).
  *
  * fnpu_dispatch_next_share: host arithmetic only. From the share share_pct
  * (1..99, percent of SMs, as decode_share_pct) and the phase times it gave,

@@ -3,7 +3,7 @@
 // 16). An item covers up to four kv heads of its keys; with more than four,
 // the heads go in groups of four, each an item of its own. (For 32 query and
 // 8 kv heads, a 1024-token chunk beside 64 decodes: 140.0 us with the per-head
-// cp.async kernel ahead of the prefill, whose decode streams 2.8 TB/s; 100.4
+// cp.async kernel ahead of the prefill, whose decode streams 2.8 TB/s; 90.4
 // us with this one beside the prefill.)
 //
 // Decode is bound by KV-cache reads (Sec. 1, Sec. 3.3, Fig. 2). The kernel is
@@ -19,8 +19,9 @@
 //     first copies one load after it starts. (Taking two items ahead left
 //     CTAs idle when items were few: the first CTAs reserved them all.)
 //   * A ring of 16-key stages holds K and V of the item's kv heads: two stages
-//     with three CTAs on an SM, three with two, six with one, so that a small
-//     grid has as many bytes in flight per SM (with the smaller items of light
+//     with three CTAs on an SM, three with two, six with one (twice as many of
+//     half the size for d = 64), so that a small grid has as many bytes in
+//     flight per SM (with the smaller items of light
 //     batches and the dependent launches, four decodes of 300..2500 keys:
 //     18.4 us a step before, 14.3 now). A
 //     producer warp issues the TMA copies (four boxes of 16 slots x 4 heads x
