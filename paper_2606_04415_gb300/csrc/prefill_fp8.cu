@@ -326,9 +326,9 @@ __device__ __forceinline__ void fp8_dequant_head(const uint8_t *__restrict__ kp,
 
 // The staging in one launch: CTAs below 4 num_jobs dequantise one kv head of
 // one block each, the others convert the queries bf16 -> f16, 8 values per load
-// and kQUnroll loads in flight a thread. Latency-bound: 128 blocks and 2176
-// tokens of 28 heads took 12.5 us with one CTA per block, its loads one after
-// another, and one load in flight a thread; 10.4 us so (34 MB, from a cold L2).
+// and kQUnroll loads in flight a thread. 563 blocks and 2176 tokens of 28
+// heads took 12.5 us with one CTA per block, its loads one after another, and one
+// load in flight a thread; 10.4 us so (59 MB from a cold L2, 8.7 at the copy rate).
 constexpr int kQUnroll = 4;
 __global__ void __launch_bounds__(128) fp8_stage_kernel(const uint8_t *__restrict__ kp, const uint8_t *__restrict__ vp,
                                                         const Fp8StageJob *__restrict__ jobs, int32_t num_jobs,
