@@ -861,22 +861,26 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
         const int64_t half_mean = (tiles + 2LL * sms - 1) / (2LL * sms);
         // Pieces of 5 or 8 tiles where a light step's few long tokens would
         // otherwise be its length: while all items together fit one wave, or
-        // the pieces half of one beside short items, and a piece is at least 6
+        // the pieces half of one beside short items whose own work (an item's
+        // switch is about 3 tiles) ends 6 tiles sooner, and a piece is at least 6
         // tiles shorter than the longest token (the merge launch costs 2 us).
         // One decode of 4001 keys 26.6 us a step with 5, 29.2 with 8, 39.0
         // with 16; 4 of 8001 48.6, 35.3 and 40.8 (208, 128 and 64 items); 126
-        // of 27..951 beside 39 prompt tokens 72.6, 72.6 and 48.9.
+        // of 27..951 beside 39 prompt tokens 72.6, 72.6 and 48.9; 12 of 410..680
+        // beside 172 prompt tokens 41.3 with 5, 33.9 with 16.
         int64_t least = 16;
         for (int64_t m : {8, 5}) {
-            int64_t items = 0, pieces = 0, longest = 0;
+            int64_t items = 0, pieces = 0, longest = 0, work = 0;
             for (int32_t s = 0; s < num_seqs; ++s)
                 for (int32_t i = 0; i < query_len[s]; ++i) {
                     const int64_t nt = (context_len[s] - query_len[s] + i + kt) / kt, ns = (nt + m - 1) / m;
                     items += 2 * ns;
                     if (ns > 1) pieces += 2 * ns;
                     longest = std::max(longest, nt);
+                    work += 2 * (nt + 3);
                 }
-            if ((items <= sms || 2 * pieces <= sms) && longest >= m + 6) least = m;
+            const bool binds = longest + 3 >= work / sms + 6;
+            if ((items <= sms || (2 * pieces <= sms && binds)) && longest >= m + 6) least = m;
         }
         mla_split_tiles = static_cast<int32_t>(std::min<int64_t>(std::max(half_mean, least), 1 << 20));
     } else if (pl->use_mla) {
