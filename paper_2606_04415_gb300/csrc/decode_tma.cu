@@ -75,8 +75,15 @@ struct DtCfg {
     static constexpr int kBarOff = kStages * kStageBytes;
     // full[S] empty[S]
     static constexpr int kNumBars = 2 * kStages;
-    // + item ring [4] and the abort flag
-    static constexpr int kSmemBytes = kBarOff + 8 * kNumBars + 32;
+    // Item ring: entry (k + 1) % kRing gets the index of item k + 1 before the
+    // producer waits for a free stage. Until then it knows of S stages less than
+    // it has issued that they were read, and an item may be a single stage, so
+    // the item whose entry it overwrites must be S + 1 items back (and entry 0
+    // of the first item, which is read ahead of any stage, S + 2). With four
+    // entries under four stages a slow warp could find a later item's index.
+    static constexpr int kRing = kStages <= 2 ? 4 : kStages <= 6 ? 8 : 16;
+    static_assert(kRing >= kStages + 2 && (kRing & (kRing - 1)) == 0, "item ring");
+    static constexpr int kSmemBytes = kBarOff + 8 * kNumBars + 4 * (kRing + 1);  // + the abort flag
 };
 
 struct DtMaps {
@@ -133,8 +140,8 @@ __global__ void __launch_bounds__(kThreads, 3)
     const uint32_t s_bars = s_base + Cfg::kBarOff;
     auto FULL = [&](int s) { return s_bars + 8 * s; };
     auto EMPTY = [&](int s) { return s_bars + 8 * (kStages + s); };
-    int *ring = reinterpret_cast<int *>(smem + Cfg::kBarOff + 8 * Cfg::kNumBars);  // [4]
-    volatile int *abort_flag = ring + 4;
+    int *ring = reinterpret_cast<int *>(smem + Cfg::kBarOff + 8 * Cfg::kNumBars);  // [kRing]
+    volatile int *abort_flag = ring + Cfg::kRing;
     int *sched = p.sched + 2;  // this kernel's work queue: next item, finished CTAs
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -300,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 3)
                 if (i == spub) {
                     if (kNoPlan && lane == 0) a = noplan_next(idx + static_cast<int>(gridDim.x));
                     idx_n = __shfl_sync(0xffffffffu, a, 0);
-                    if (lane == 0) *reinterpret_cast<volatile int *>(ring + ((k + 1) & 3)) = idx_n;
+                    if (lane == 0) *reinterpret_cast<volatile int *>(ring + ((k + 1) & (Cfg::kRing - 1))) = idx_n;
                     __syncwarp();  // before the arrival of this stage, which releases it
                     if (idx_n < n_items) nit = item_at(idx_n);
                 }
@@ -344,7 +351,7 @@ __global__ void __launch_bounds__(kThreads, 3)
                 const int st = gs % kStages;
                 if (!wait(FULL(st), (gs / kStages) & 1)) { ok = false; break; }
                 if (i == spub) {  // the producer published it before issuing this stage
-                    idx_n = *reinterpret_cast<volatile int *>(ring + ((k + 1) & 3));
+                    idx_n = *reinterpret_cast<volatile int *>(ring + ((k + 1) & (Cfg::kRing - 1)));
                     has_next = idx_n < n_items;
                     if (has_next) nit = item_at(idx_n);
                 }

@@ -755,3 +755,25 @@ def test_qwen_coloc_other_seeds_sampled_rows(seed):
     st = _step(batch)
     out, lse = st.results()
     _compare(batch, out, lse, tokens=_sample_tokens(batch, per_seq_rows=6, seed=seed))
+
+
+@pytest.mark.parametrize("beside", [False, True])
+@pytest.mark.parametrize("dim", [64, 128])
+def test_many_decodes_of_a_stage_or_three(dim, beside):
+    """Far more items than CTAs, of one 16-key stage after a few of three, so that
+    each CTA's ring of item indices turns several times while its stages are few
+    items apart: every row right, and the same bits again, alone and beside a
+    prefill chunk."""
+    sh = W.Shape(4, 2, dim, dim, 16, False)
+    rng = np.random.default_rng(dim)
+    ctx = np.concatenate([rng.integers(33, 49, size=400), rng.integers(1, 17, size=3000)])
+    rng.shuffle(ctx)
+    ql, c, ph = ([300], [1500], [0]) if beside else ([], [], [])
+    batch = W.build_batch(sh, ql + [1] * len(ctx), c + ctx.tolist(), ph + [1] * len(ctx), rng, name="short_items")
+    st = _step(batch, share=50 if beside else 0)
+    out, lse = st.results()
+    _compare(batch, out, lse)
+    for _ in range(5):
+        st.run()
+        out2, lse2 = st.results()
+        assert np.array_equal(out, out2) and np.array_equal(lse, lse2)

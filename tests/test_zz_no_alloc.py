@@ -192,3 +192,31 @@ def test_noalloc_head_groups_block_sizes_and_split_lengths(heads, bs, split_keys
     ref_o, ref_l = _oracle_after_append(batch)
     assert np.abs(out.float().cpu().numpy() - ref_o).max() <= O_TOL
     assert np.abs(lse.cpu().numpy() - ref_l).max() <= LSE_TOL
+
+
+@pytest.mark.parametrize("dim", [64, 128])
+def test_noalloc_many_sequences_of_a_stage_or_three(dim):
+    """Several items a CTA, most of one 16-key stage (as the planned decode's test
+    of the item ring): every row right, and the same bits again."""
+    _need_gpu()
+    import paper_2606_04415_gb300 as fnpu
+    from paper_2606_04415_gb300.step import DeviceStep
+    sh = W.Shape(4, 2, dim, dim, 16, False)
+    rng = np.random.default_rng(dim + 1)
+    ctx = np.concatenate([rng.integers(33, 49, size=400), rng.integers(1, 17, size=3000)])
+    batch = W.build_batch(sh, np.ones_like(ctx), ctx, np.ones(len(ctx), np.uint8), rng, name="noalloc_short")
+    st = DeviceStep(batch)
+    st.append()
+    ref_o, ref_l = _oracle_after_append(batch)
+    dctx, bt = torch.from_numpy(batch.context_len).cuda(), torch.from_numpy(batch.block_table).cuda()
+    first = None
+    for call in range(5):
+        out, lse = torch.full_like(st.out, float("nan")), torch.full_like(st.lse, float("nan"))
+        fnpu.decode_attn_noalloc(st.desc, dctx, bt, 48, st.q, st.k_cache, st.v_cache, out, lse)
+        torch.cuda.synchronize()
+        o, l = out.float().cpu().numpy(), lse.cpu().numpy()
+        if first is None:
+            first = o, l
+            assert np.abs(o - ref_o).max() <= O_TOL and np.abs(l - ref_l).max() <= LSE_TOL
+        assert np.array_equal(o, first[0]) and np.array_equal(l, first[1]), f"call {call}"
+    assert fnpu.check() == fnpu.FNPU_OK
