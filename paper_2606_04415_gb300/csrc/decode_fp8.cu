@@ -53,7 +53,12 @@ constexpr int kStageBytes = 2 * kCodeBytes + 2 * kScaleBytes;  // K codes, V cod
 constexpr int kStageStride = (kStageBytes + 1023) / 1024 * 1024;  // the swizzled K codes need 1024-byte alignment
 constexpr int kBarOff = kStages * kStageStride;
 constexpr int kNumBars = 2 * kStages;
-constexpr int kSmemBytes = kBarOff + 8 * kNumBars + 32;  // + item ring [4] and the abort flag
+// Item ring: written before the producer waits for a free stage, so an entry is
+// used again S + 2 items later at the soonest (as in the bf16 kernel; items of a
+// single block with four entries let a slow warp find a later item's index).
+constexpr int kRing = 8;
+static_assert(kRing >= kStages + 2 && (kRing & (kRing - 1)) == 0, "item ring");
+constexpr int kSmemBytes = kBarOff + 8 * kNumBars + 4 * (kRing + 1);  // + the abort flag
 static_assert(kCodeBytes % 1024 == 0 && kStageStride % 1024 == 0, "swizzle atoms");
 
 struct Fp8Maps {
@@ -98,8 +103,8 @@ __global__ void __launch_bounds__(kThreads, 3)
     const uint32_t s_bars = s_base + kBarOff;
     auto FULL = [&](int s) { return s_bars + 8 * s; };
     auto EMPTY = [&](int s) { return s_bars + 8 * (kStages + s); };
-    int *ring = reinterpret_cast<int *>(smem + kBarOff + 8 * kNumBars);  // [4]
-    volatile int *abort_flag = ring + 4;
+    int *ring = reinterpret_cast<int *>(smem + kBarOff + 8 * kNumBars);  // [kRing]
+    volatile int *abort_flag = ring + kRing;
     int *sched = p.sched + 2;  // the decode work queue: next item, finished CTAs
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -205,7 +210,7 @@ __global__ void __launch_bounds__(kThreads, 3)
             for (int i = 0; i < ntiles; ++i, ++gs) {
                 if (i == spub) {
                     idx_n = __shfl_sync(0xffffffffu, a, 0);
-                    if (lane == 0) *reinterpret_cast<volatile int *>(ring + ((k + 1) & 3)) = idx_n;
+                    if (lane == 0) *reinterpret_cast<volatile int *>(ring + ((k + 1) & (kRing - 1))) = idx_n;
                     __syncwarp();  // before the arrival of this stage, which releases it
                     if (idx_n < n_items) nit = p.ditems[idx_n];
                 }
@@ -252,7 +257,7 @@ __global__ void __launch_bounds__(kThreads, 3)
                 const int st = gs % kStages;
                 if (!wait(FULL(st), (gs / kStages) & 1)) { ok = false; break; }
                 if (i == spub) {  // the producer published it before issuing this stage
-                    idx_n = *reinterpret_cast<volatile int *>(ring + ((k + 1) & 3));
+                    idx_n = *reinterpret_cast<volatile int *>(ring + ((k + 1) & (kRing - 1)));
                     has_next = idx_n < n_items;
                     if (has_next) nit = p.ditems[idx_n];
                 }

@@ -309,3 +309,24 @@ def test_fp8_random_mixed_step_all_rows(case):
     flags = int(rng.choice([0, 0, 0, 1, 2]))  # separate launches / the mma.sync prefill
     _, out, lse, kp, vp = _run(batch, seed=70 + case, split=split, flags=flags, share=share)
     _compare(batch, out, lse, kp, vp)
+
+
+@pytest.mark.parametrize("beside", [False, True])
+def test_fp8_many_decodes_of_a_block_or_three(beside):
+    """Far more items than CTAs, of one block after a few of three, so that each
+    CTA's ring of item indices turns several times while its stages are few items
+    apart: every row right, and the same bits again, alone and beside a chunk."""
+    rng = np.random.default_rng(8)
+    ctx = np.concatenate([rng.integers(33, 49, size=300), rng.integers(1, 17, size=3000)])
+    rng.shuffle(ctx)
+    n = len(ctx)
+    if beside:
+        batch = _batch([900] + ctx.tolist(), seed=9, ql=[200] + [1] * n, phase=[0] + [1] * n)
+    else:
+        batch = _batch(ctx, seed=9)
+    st, out, lse, kp, vp = _run(batch, check_pools=False, share=50 if beside else 0)
+    _compare(batch, out, lse, kp, vp)
+    for _ in range(5):
+        st.run()
+        out2, lse2 = st.results()
+        assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
