@@ -635,9 +635,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!wait(MLX, nd & 1) || !wait(ODONE(1 - w), k & 1)) break;
                 tc::fence_after_sync();
                 const float2 a = ml[r], b = ml[128 + r];
-                const bool va = a.y > 0.f, vb = b.y > 0.f;
-                const float M = fmaxf(va ? a.x : -INFINITY, vb ? b.x : -INFINITY);
-                const float fa = va ? fast_exp2(a.x - M) : 0.f, fb = vb ? fast_exp2(b.x - M) : 0.f;
+                // A sum of zero: no key of the path is visible to the row (its O may
+                // hold 0 * NaN and is left out). Any other sum counts, NaN
+                // included, and so do two sums of zero (all scores -inf).
+                const bool va = a.y != 0.f || b.y == 0.f, vb = b.y != 0.f || a.y == 0.f;
+                const float M = fmaxf(a.x, b.x);  // (-inf on a path without a key)
+                const float fa = a.y != 0.f ? fast_exp2(a.x - M) : 0.f, fb = b.y != 0.f ? fast_exp2(b.x - M) : 0.f;
                 const float L = a.y * fa + b.y * fb, iL = 1.f / L;
                 const float ca = fa * iL, cb = fb * iL;
                 const int64_t prow = (static_cast<int64_t>(it.pbase + it.split) * 2) * 128;

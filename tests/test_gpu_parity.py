@@ -777,3 +777,33 @@ def test_many_decodes_of_a_stage_or_three(dim, beside):
         st.run()
         out2, lse2 = st.results()
         assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
+
+
+@pytest.mark.parametrize("ctx", [1500, 9000])
+@pytest.mark.parametrize("what", ["nan query", "inf query", "nan key, odd tile", "nan key, even tile"])
+def test_nan_and_infinity_reach_their_rows_through_single_q_tile_items(what, ctx):
+    """A chunk of one Q tile merges two softmax paths, of which one may have seen
+    no key of a row. A NaN or infinite query, or a NaN key on one path, is
+    something else: it makes NaN of the rows that see it, unsplit and with key
+    splits (9000 keys on 12 SMs), and leaves all others as they are."""
+    import paper_2606_04415_gb300 as fnpu
+    from paper_2606_04415_gb300.step import DeviceStep
+    sh = W.SHAPES["qwen"]
+    batch = W.build_batch(sh, [4, 18, 3], [ctx, 1300, 700], [1, 1, 1], np.random.default_rng(ctx), name="one_tile_nan")
+    ref_o, ref_l, _, _ = oracle.run_step(batch)
+    bad = np.zeros(ref_l.shape, bool)  # (token, head) rows that meet it
+    if what.endswith("query"):
+        batch.q[1, 5, 7] = 0x7FC0 if what == "nan query" else 0x7F80
+        bad[1, 5] = True
+    else:
+        key = 128 * 3 + 5 if "odd" in what else 128 * 2 + 5  # of sequence 0, whose new rows all come later
+        batch.k_cache[batch.block_table[0, key // 16], key % 16, 2, 9] = 0x7FC0
+        bad[:4, 14:21] = True  # the query heads of kv head 2
+    st = DeviceStep(batch, opts=fnpu.PlanOpts(0, 0, 12, 0))
+    assert st.plan.info()["prefill_items"] == 12 if ctx == 1500 else st.plan.info()["prefill_items"] > 12
+    st.run()
+    out, lse = st.results()
+    assert fnpu.plan_check(st.plan) == fnpu.FNPU_OK
+    assert np.isnan(out[bad]).all() and np.isnan(lse[bad]).all()
+    assert np.isfinite(out[~bad]).all() and np.isfinite(lse[~bad]).all()
+    assert np.abs(out - ref_o)[~bad].max() <= O_TOL and np.abs(lse - ref_l)[~bad].max() <= LSE_TOL
