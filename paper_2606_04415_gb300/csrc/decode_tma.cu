@@ -122,6 +122,11 @@ __device__ __forceinline__ void load_q(const AttnParams &p, int t, int head, int
     }
 }
 
+// what the bf16 pair `r` leaves of the values it was rounded from
+__device__ __forceinline__ uint32_t bf16x2_rest(uint32_t r, float lo, float hi) {
+    return pack_bf16x2(lo - __uint_as_float(r << 16), hi - __uint_as_float(r & 0xFFFF0000u));
+}
+
 // block ids of the item's blocks, relative block `lane` in lane `lane`
 __device__ __forceinline__ int load_blk_lane(const AttnParams &p, const DtGeo &g, int lane) {
     const int b0 = g.kb / p.block_size;
@@ -131,7 +136,15 @@ __device__ __forceinline__ int load_blk_lane(const AttnParams &p, const DtGeo &g
 
 // kRagged: the kv heads are no multiple of four, so that a warp of the last
 // group may have none (the checks cost a small step 7% where they are not needed)
-template <int D, bool kRagged, int kStages, bool kNoPlan>
+// kFineP: P enters its product as two bf16 operands, its rounding and the rest.
+// Where this kernel took the place of the per-head ones (without a plan, and for
+// other than four kv heads) they had a running maximum per warp and quarter of a
+// 64-key tile, so that more probabilities were exactly 1 before they were
+// rounded: 1.73e-3 off the 64-bit result without a plan (16 sequences, 32/8
+// heads) and 1.77e-3 with one (64), where one operand gives 1.81e-3 and 1.83e-3
+// and two 1.64e-3 and 1.66e-3. They cost 43.1 -> 44.7 us of that call, and a
+// light step of four kv heads, which always had one, would pay 14.3 -> 15.0.
+template <int D, bool kRagged, int kStages, bool kNoPlan, bool kFineP>
 __global__ void __launch_bounds__(kThreads, 3)
     decode_tma_kernel(const AttnParams p, const __grid_constant__ DtMaps maps) {
     using Cfg = DtCfg<D, kStages>;
@@ -397,13 +410,19 @@ __global__ void __launch_bounds__(kThreads, 3)
                 for (int mt = 0; mt < D / 16; ++mt) {
                     o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
                 }
-                const uint32_t pb0 = movmatrix_trans(pack_bf16x2(p0, p1));
-                const uint32_t pb1 = movmatrix_trans(pack_bf16x2(p2, p3));
+                const uint32_t r01 = pack_bf16x2(p0, p1), r23 = pack_bf16x2(p2, p3);
+                const uint32_t pb0 = movmatrix_trans(r01), pb1 = movmatrix_trans(r23);
+                uint32_t pe0 = 0u, pe1 = 0u;
+                if constexpr (kFineP) {
+                    pe0 = movmatrix_trans(bf16x2_rest(r01, p0, p1));
+                    pe1 = movmatrix_trans(bf16x2_rest(r23, p2, p3));
+                }
 #pragma unroll
                 for (int mt = 0; mt < D / 16; ++mt) {
                     uint32_t a0, a1, a2, a3;
                     ldmatrix_x4_trans(a0, a1, a2, a3, sV + dt_off(lr + 8 * (lj >> 1), wh, 2 * mt + (lj & 1)));
                     mma_bf16_16816(o[mt], a0, a1, a2, a3, pb0, pb1);
+                    if constexpr (kFineP) mma_bf16_16816(o[mt], a0, a1, a2, a3, pe0, pe1);
                 }
                 if (tail) tc::fence_proxy_async_smem();  // order the zeroing before the next TMA write
                 }
@@ -595,10 +614,10 @@ bool encode_slot_major_map(CUtensorMap *m, const void *base, int d, int hkv, int
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, bool kRagged, int kStages, bool kNoPlan>
+template <int D, bool kRagged, int kStages, bool kNoPlan, bool kFineP>
 int launch_dt(const AttnParams &p, cudaStream_t st, int grid, bool after_prev) {
     using Cfg = DtCfg<D, kStages>;
-    auto kernel = decode_tma_kernel<D, kRagged, kStages, kNoPlan>;
+    auto kernel = decode_tma_kernel<D, kRagged, kStages, kNoPlan, kFineP>;
     DtMaps maps;
     if (!encode_slot_major_map(&maps.k, p.k_cache, D, p.num_kv_heads, p.block_size, p.num_blocks) ||
         !encode_slot_major_map(&maps.v, p.v_cache, D, p.num_kv_heads, p.block_size, p.num_blocks))
@@ -614,26 +633,28 @@ int launch_dt(const AttnParams &p, cudaStream_t st, int grid, bool after_prev) {
 // for d = 64), and all of them should be in flight whatever the number of CTAs on
 // it (d = 64, 2 kv heads, 64 decodes of 500..4000 keys: 28.2 us a step with half
 // of them, 24.3 with all).
-template <int D, bool kRagged, bool kNoPlan>
+template <int D, bool kRagged, bool kNoPlan, bool kFineP>
 int launch_dt(const AttnParams &p, cudaStream_t st, int max_ctas, bool alone) {
     const int grid = p.num_ditems < max_ctas ? p.num_ditems : max_ctas;
     const int sms = max_ctas / 3;
     constexpr int k = 128 / D;  // (stages of 16 KB for d = 64)
-    if (alone && grid <= sms) return launch_dt<D, kRagged, 6 * k, kNoPlan>(p, st, grid, alone);
-    if (alone && grid <= 2 * sms) return launch_dt<D, kRagged, 3 * k, kNoPlan>(p, st, grid, alone);
-    return launch_dt<D, kRagged, 2 * k, kNoPlan>(p, st, grid, alone);
+    if (alone && grid <= sms) return launch_dt<D, kRagged, 6 * k, kNoPlan, kFineP>(p, st, grid, alone);
+    if (alone && grid <= 2 * sms) return launch_dt<D, kRagged, 3 * k, kNoPlan, kFineP>(p, st, grid, alone);
+    return launch_dt<D, kRagged, 2 * k, kNoPlan, kFineP>(p, st, grid, alone);
+}
+
+template <int D, bool kNoPlan>
+int launch_dt_heads(const AttnParams &p, cudaStream_t st, int max_ctas, bool alone) {
+    if (p.num_kv_heads % kHkv != 0) return launch_dt<D, true, kNoPlan, true>(p, st, max_ctas, alone);
+    if (kNoPlan || p.num_kv_heads != 4) return launch_dt<D, false, kNoPlan, true>(p, st, max_ctas, alone);
+    return launch_dt<D, false, kNoPlan, kNoPlan>(p, st, max_ctas, alone);
 }
 
 template <bool kNoPlan>
 int launch_dt_shape(const AttnParams &p, cudaStream_t st, int max_ctas, bool alone) {
-    const bool ragged = p.num_kv_heads % kHkv != 0;
     switch (p.head_dim_qk) {
-        case 64:
-            return ragged ? launch_dt<64, true, kNoPlan>(p, st, max_ctas, alone)
-                          : launch_dt<64, false, kNoPlan>(p, st, max_ctas, alone);
-        case 128:
-            return ragged ? launch_dt<128, true, kNoPlan>(p, st, max_ctas, alone)
-                          : launch_dt<128, false, kNoPlan>(p, st, max_ctas, alone);
+        case 64: return launch_dt_heads<64, kNoPlan>(p, st, max_ctas, alone);
+        case 128: return launch_dt_heads<128, kNoPlan>(p, st, max_ctas, alone);
         default: return FNPU_EUNSUPPORTED;
     }
 }

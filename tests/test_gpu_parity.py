@@ -807,3 +807,18 @@ def test_nan_and_infinity_reach_their_rows_through_single_q_tile_items(what, ctx
     assert np.isnan(out[bad]).all() and np.isnan(lse[bad]).all()
     assert np.isfinite(out[~bad]).all() and np.isfinite(lse[~bad]).all()
     assert np.abs(out - ref_o)[~bad].max() <= O_TOL and np.abs(lse - ref_l)[~bad].max() <= LSE_TOL
+
+
+@pytest.mark.parametrize("heads,dim", [((32, 8), 128), ((4, 2), 64), ((6, 3), 128)])
+def test_decode_probabilities_lose_nothing_to_bf16(heads, dim):
+    """Other than four kv heads: the probabilities enter their product as two bf16
+    operands, so that a result is off by little more than its own rounding (2^-16
+    of a probability is left out, and fp32 sums err by less; one operand, at
+    2^-9, would add about as much again as the rounding)."""
+    sh = W.Shape(*heads, dim, dim, 16, False)
+    ctx = [700, 1500, 333, 2048, 64]
+    batch = W.build_batch(sh, [1] * len(ctx), ctx, [1] * len(ctx), np.random.default_rng(dim), name="fine_p")
+    out, _ = _step(batch).results()
+    ref, _, _, _ = oracle.run_step(batch)
+    rounded = W.bf16_bits_to_f32(W.f32_to_bf16_bits(ref))
+    assert np.linalg.norm(out - ref) <= 1.05 * np.linalg.norm(rounded - ref)

@@ -220,3 +220,23 @@ def test_noalloc_many_sequences_of_a_stage_or_three(dim):
             assert np.abs(o - ref_o).max() <= O_TOL and np.abs(l - ref_l).max() <= LSE_TOL
         assert np.array_equal(o, first[0]) and np.array_equal(l, first[1]), f"call {call}"
     assert fnpu.check() == fnpu.FNPU_OK
+
+
+@pytest.mark.parametrize("heads,dim", [((32, 8), 128), ((28, 4), 128), ((4, 2), 64)])
+def test_noalloc_probabilities_lose_nothing_to_bf16(heads, dim):
+    """As the planned decode's test of the same name: a result is off by little
+    more than its own rounding to bf16."""
+    _need_gpu()
+    import paper_2606_04415_gb300 as fnpu
+    from paper_2606_04415_gb300.step import DeviceStep
+    sh = W.Shape(*heads, dim, dim, 16, False)
+    ctx = [700, 1500, 333, 2048, 64]
+    batch = W.build_batch(sh, [1] * len(ctx), ctx, [1] * len(ctx), np.random.default_rng(dim), name="fine_p")
+    st = DeviceStep(batch)
+    st.append()
+    fnpu.decode_attn_noalloc(st.desc, torch.from_numpy(batch.context_len).cuda(), torch.from_numpy(batch.block_table).cuda(),
+                             max(ctx), st.q, st.k_cache, st.v_cache, st.out, st.lse)
+    out, _ = st.results()
+    ref, _ = _oracle_after_append(batch)
+    rounded = W.bf16_bits_to_f32(W.f32_to_bf16_bits(ref))
+    assert np.linalg.norm(out - ref) <= 1.05 * np.linalg.norm(rounded - ref)
