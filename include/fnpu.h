@@ -334,8 +334,10 @@ int fnpu_plan_decode_share(const fnpu_plan *plan, int32_t *share_pct);
  * the FP8 cache (kv_fp8 = 1: plan-based runs only);
  * FNPU_ECUDA. Nothing is launched on error.
  * The first call on a device looks up the scratch array's device address
- * (cudaGetSymbolAddress) while that device is current; make that first call
- * before any stream capture. All calls share the one array, which keeps the
+ * (cudaGetSymbolAddress) while that device is current, and loads the code of
+ * every kernel that a call may come to, whatever its shape and batch; make
+ * that first call before any stream capture, and before device memory is full.
+ * Later calls load nothing and may be captured. All calls share the one array, which keeps the
  * last call's contents; a call that merges by counters (block sizes that are
  * no multiple of 16) clears them itself with cudaMemsetAsync on `stream`. Calls that overlap on the GPU (on different
  * streams, or with no ordering between them) race on the array and must not

@@ -285,8 +285,16 @@ __global__ void __launch_bounds__(kThreads, 2) decode_noalloc_kernel(const Noall
 std::mutex g_setup_mu;
 float *g_scratch_addr[kMaxDevices] = {};
 
+template <int D>
+int prepare_noalloc() {  // (setting the attribute also loads the kernel's code)
+    FNPU_CUDA_TRY(cudaFuncSetAttribute(decode_noalloc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kStages * 2 * kTileKeys * D * 2));
+    return FNPU_OK;
+}
+
 // Device address of g_noalloc_scratch on the current device, looked up once
-// per device (the first call on a device does it; see fnpu.h).
+// per device; that first call also loads the code of every kernel that a later
+// one may come to, so that none is loaded then (see fnpu.h).
 int scratch_address(float **out) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return FNPU_ECUDA;
@@ -298,6 +306,8 @@ int scratch_address(float **out) {
             cudaGetLastError();
             return FNPU_ECUDA;
         }
+        for (int rc : {prepare_decode_tma_noplan(), prepare_noalloc<64>(), prepare_noalloc<128>()})
+            if (rc != FNPU_OK) return rc;
         g_scratch_addr[dev] = static_cast<float *>(ptr);
     }
     *out = g_scratch_addr[dev];
@@ -307,9 +317,8 @@ int scratch_address(float **out) {
 template <int D>
 int launch_noalloc(const NoallocParams &p, int grid, cudaStream_t st) {
     constexpr int kSmem = kStages * 2 * kTileKeys * D * 2;
-    if (cudaFuncSetAttribute(decode_noalloc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kSmem) != cudaSuccess)
-        return FNPU_ECUDA;
+    const int rc = prepare_noalloc<D>();
+    if (rc != FNPU_OK) return rc;
     decode_noalloc_kernel<D><<<grid, kThreads, kSmem, st>>>(p);
     return cudaGetLastError() == cudaSuccess ? FNPU_OK : FNPU_ECUDA;
 }

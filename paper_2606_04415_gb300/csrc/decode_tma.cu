@@ -614,6 +614,17 @@ bool encode_slot_major_map(CUtensorMap *m, const void *base, int d, int hkv, int
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// (setting an attribute also loads the kernel's code)
+template <int D, bool kRagged, int kStages, bool kNoPlan, bool kFineP>
+int prepare_dt() {
+    auto kernel = decode_tma_kernel<D, kRagged, kStages, kNoPlan, kFineP>;
+    FNPU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       DtCfg<D, kStages>::kSmemBytes));
+    FNPU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                       cudaSharedmemCarveoutMaxShared));
+    return FNPU_OK;
+}
+
 template <int D, bool kRagged, int kStages, bool kNoPlan, bool kFineP>
 int launch_dt(const AttnParams &p, cudaStream_t st, int grid, bool after_prev) {
     using Cfg = DtCfg<D, kStages>;
@@ -622,9 +633,8 @@ int launch_dt(const AttnParams &p, cudaStream_t st, int grid, bool after_prev) {
     if (!encode_slot_major_map(&maps.k, p.k_cache, D, p.num_kv_heads, p.block_size, p.num_blocks) ||
         !encode_slot_major_map(&maps.v, p.v_cache, D, p.num_kv_heads, p.block_size, p.num_blocks))
         return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled (decode)");
-    FNPU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
-    FNPU_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                       cudaSharedmemCarveoutMaxShared));
+    const int rc = prepare_dt<D, kRagged, kStages, kNoPlan, kFineP>();
+    if (rc != FNPU_OK) return rc;
     FNPU_CUDA_TRY(launch_ex(kernel, grid, kThreads, Cfg::kSmemBytes, st, after_prev, nullptr, p, maps));
     return FNPU_OK;
 }
@@ -641,6 +651,19 @@ int launch_dt(const AttnParams &p, cudaStream_t st, int max_ctas, bool alone) {
     if (alone && grid <= sms) return launch_dt<D, kRagged, 6 * k, kNoPlan, kFineP>(p, st, grid, alone);
     if (alone && grid <= 2 * sms) return launch_dt<D, kRagged, 3 * k, kNoPlan, kFineP>(p, st, grid, alone);
     return launch_dt<D, kRagged, 2 * k, kNoPlan, kFineP>(p, st, grid, alone);
+}
+
+// every kernel that a call without a plan may come to for head width D
+template <int D>
+int prepare_noplan() {
+    constexpr int k = 128 / D;
+    for (int rc : {prepare_dt<D, true, 2 * k, true, true>(), prepare_dt<D, true, 3 * k, true, true>(),
+                   prepare_dt<D, true, 6 * k, true, true>(), prepare_dt<D, false, 2 * k, true, true>(),
+                   prepare_dt<D, false, 3 * k, true, true>(), prepare_dt<D, false, 6 * k, true, true>()})
+        if (rc != FNPU_OK) return rc;
+    cudaFuncAttributes a;
+    FNPU_CUDA_TRY(cudaFuncGetAttributes(&a, split_merge_kernel<D, true>));
+    return FNPU_OK;
 }
 
 template <int D, bool kNoPlan>
@@ -690,6 +713,11 @@ int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas, bool alon
     const int rc = launch_dt_shape<false>(p, static_cast<cudaStream_t>(stream), max_ctas, alone);
     if (rc != FNPU_OK) return rc;
     return launch_split_merge(p, stream);
+}
+
+int prepare_decode_tma_noplan() {
+    const int rc = prepare_noplan<64>();
+    return rc != FNPU_OK ? rc : prepare_noplan<128>();
 }
 
 int launch_decode_tma_noplan(const AttnParams &p, void *stream, int max_ctas) {

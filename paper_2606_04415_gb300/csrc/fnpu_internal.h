@@ -183,6 +183,10 @@ int decode_tma_heads_per_item();
 // without a plan: p.na_*, num_ditems = sequences x head groups x na_max_splits,
 // num_mgroups = sequences, partial rows sequence x na_max_splits + split
 int launch_decode_tma_noplan(const AttnParams &p, void *stream, int max_ctas);
+// Loads every kernel that launch_decode_tma_noplan may launch on the current
+// device: which one follows from the batch, and a first use later could load
+// code under a stream capture or where no device memory may be taken.
+int prepare_decode_tma_noplan();
 int launch_prefill_mma(const AttnParams &p, void *stream);
 int launch_mla(const AttnParams &p, void *stream);
 // tcgen05 latent attention: items are (token, d_v half, key range) of 128 heads

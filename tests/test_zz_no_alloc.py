@@ -240,3 +240,60 @@ def test_noalloc_probabilities_lose_nothing_to_bf16(heads, dim):
     ref, _ = _oracle_after_append(batch)
     rounded = W.bf16_bits_to_f32(W.f32_to_bf16_bits(ref))
     assert np.linalg.norm(out - ref) <= 1.05 * np.linalg.norm(rounded - ref)
+
+
+_ONE_CALL_PREPARES = """
+import torch
+import paper_2606_04415_gb300 as fnpu
+
+def call(n, ctx, hq, hkv, d, bs=16):
+    nb = n * ((ctx + bs - 1) // bs)
+    desc = fnpu.make_desc(hq, hkv, d, d, bs, nb)
+    cl = torch.full((n,), ctx, dtype=torch.int32, device="cuda")
+    bt = torch.arange(nb, dtype=torch.int32, device="cuda").view(n, -1)
+    q = torch.randn(n, hq, d, device="cuda").bfloat16()
+    k, v = (torch.randn(nb, bs, hkv, d, device="cuda").bfloat16() for _ in range(2))
+    out, lse = torch.empty_like(q), torch.empty(n, hq, device="cuda")
+    return (lambda: fnpu.decode_attn_noalloc(desc, cl, bt, ctx, q, k, v, out, lse)), out, lse
+
+small = call(1, 16, 4, 2, 64)
+others = [call(n, ctx, hq, hkv, d, bs) for hq, hkv, d, bs in
+          [(32, 8, 128, 16), (9, 3, 128, 16), (4, 4, 64, 16), (6, 2, 64, 16), (28, 4, 128, 24), (4, 4, 64, 24)]
+          for n, ctx in [(1, 60), (1, 5000), (20, 2000), (60, 4000)]]
+torch.cuda.synchronize()
+small[0]()
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+for f, out, lse in others[::2]:
+    f()
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] == free
+for f, out, lse in others:
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        f()
+    g.replay()
+    torch.cuda.synchronize()
+    a = out.clone(), lse.clone()
+    out.fill_(float("nan"))
+    lse.fill_(float("nan"))
+    f()
+    torch.cuda.synchronize()
+    assert torch.equal(a[0], out) and torch.equal(a[1], lse)
+    assert torch.isfinite(out).all() and torch.isfinite(lse).all()
+assert fnpu.check() == fnpu.FNPU_OK
+print("prepared")
+"""
+
+
+def test_noalloc_one_call_prepares_all_later_ones():
+    """In a fresh process, one small call; after it no call takes device memory,
+    and every other head shape, ring depth and merge (half of them not called
+    before) is captured into a graph and replayed, with a direct call's results."""
+    _need_gpu()
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _ONE_CALL_PREPARES], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "prepared" in r.stdout, r.stdout + r.stderr
