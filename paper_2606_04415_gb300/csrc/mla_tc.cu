@@ -81,8 +81,8 @@ constexpr int kOffStage = kOffV + kStages * kVBytes;  // a 32-row x 64-column bo
 constexpr int kOffL = kOffStage + kQChunkBytes;       // [2 items][128 rows] (log2 max, sum)
 constexpr int kOffBar = kOffL + 2 * kRows * 8;
 // nfull[2] nempty[2] vfull[2] vempty[2] itemfull[4] itemempty[4] and
-// sfull sfree pready odone ofree lready qfull qready qfree drain stage[4]
-constexpr int kNumBars = 4 * kStages + 2 * kItemSlots + 14;
+// sfull sfree pready odone ofree lready[2] qfull qready qfree drain stage[4]
+constexpr int kNumBars = 4 * kStages + 2 * kItemSlots + 15;
 constexpr int kOffMisc = kOffBar + 8 * kNumBars;      // tmem address, abort flag, item ring
 constexpr int kSmemBytes = kOffMisc + 8 + 4 * kItemSlots;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
@@ -105,9 +105,13 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
     auto ITEMFULL = [&](int s) { return b1 + 8 * s; };
     auto ITEMEMPTY = [&](int s) { return b1 + 8 * (kItemSlots + s); };
     const uint32_t b2 = b1 + 16 * kItemSlots;
-    const uint32_t SFULL = b2, SFREE = b2 + 8, PREADY = b2 + 16, ODONE = b2 + 24, OFREE = b2 + 32, LREADY = b2 + 40,
-                   QFULL = b2 + 48, QREADY = b2 + 56, QFREE = b2 + 64, DRAIN = b2 + 72;
-    auto STAGE = [&](int w) { return b2 + 80 + 8 * w; };
+    const uint32_t SFULL = b2, SFREE = b2 + 8, PREADY = b2 + 16, ODONE = b2 + 24, OFREE = b2 + 32,
+                   QFULL = b2 + 56, QREADY = b2 + 64, QFREE = b2 + 72, DRAIN = b2 + 80;
+    // (one for even and one for odd items: an item of one tile may end before an
+    // epilogue warp has looked at the end of the one before; the next of the same
+    // parity cannot, as its Q comes from that warp)
+    auto LREADY = [&](int k) { return b2 + 40 + 8 * (k & 1); };
+    auto STAGE = [&](int w) { return b2 + 88 + 8 * w; };
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + kOffMisc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + kOffMisc + 4);
     volatile int *item_slot = reinterpret_cast<volatile int *>(smem + kOffMisc + 8);  // [kItemSlots]
@@ -136,7 +140,8 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
         tc::mbar_init(PREADY, 4);
         tc::mbar_init(ODONE, 1);
         tc::mbar_init(OFREE, 4);
-        tc::mbar_init(LREADY, 4);
+        tc::mbar_init(LREADY(0), 4);
+        tc::mbar_init(LREADY(1), 4);
         tc::mbar_init(QFULL, 1);
         tc::mbar_init(QREADY, 4);
         tc::mbar_init(QFREE, 1);
@@ -445,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
             (void)half;
             l_buf[(k & 1) * kRows + r] = make_float2(m_run, l);
             __syncwarp();
-            tc::mbar_arrive_warp(LREADY);
+            tc::mbar_arrive_warp(LREADY(k));
             tc::mbar_arrive_warp(ITEMEMPTY(k % kItemSlots));
         }
     } else {
@@ -480,7 +485,7 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
             return true;
         };
         auto epilogue = [&](const MlaItem &it, int k) -> bool {
-            if (!wait(LREADY, k & 1) || !wait(ODONE, k & 1)) return false;
+            if (!wait(LREADY(k), (k >> 1) & 1) || !wait(ODONE, k & 1)) return false;
             tc::fence_after_sync();
             const float2 ml = l_buf[(k & 1) * kRows + r];
             const float inv = 1.f / ml.y;

@@ -822,3 +822,21 @@ def test_decode_probabilities_lose_nothing_to_bf16(heads, dim):
     ref, _, _, _ = oracle.run_step(batch)
     rounded = W.bf16_bits_to_f32(W.f32_to_bf16_bits(ref))
     assert np.linalg.norm(out - ref) <= 1.05 * np.linalg.norm(rounded - ref)
+
+
+def test_mla_many_items_of_one_tile():
+    """Several one-tile items in a row on each CTA of the latent kernel, whose
+    softmax may then end an item before the epilogue of the one before has begun."""
+    sh = W.Shape(128, 1, 576, 512, 64, True)
+    rng = np.random.default_rng(64)
+    ctx = rng.integers(1, 65, size=900)
+    batch = W.build_batch(sh, [1] * len(ctx), ctx, [1] * len(ctx), rng, name="mla_one_tile")
+    st = _step(batch)
+    out, lse = st.results()
+    _compare(batch, out, lse)
+    for _ in range(10):
+        st.run()
+        out2, lse2 = st.results()
+        assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
+    import paper_2606_04415_gb300 as fnpu
+    assert fnpu.plan_check(st.plan) == fnpu.FNPU_OK
