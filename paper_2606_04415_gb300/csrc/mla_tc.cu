@@ -257,16 +257,6 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
             }
             idx = idx_n;
         }
-        if (!ok) {
-            // gave up: let the copies already issued land before the CTA
-            // leaves (bounded), so that none writes into a later CTA
-            for (int g = gt > kStages ? gt - kStages : 0; g < gt; ++g)
-                tc::mbar_wait(NFULL(g % kStages), (g / kStages) & 1, 200000000ull);
-            for (int g = gv > kStages ? gv - kStages : 0; g < gv; ++g)
-                tc::mbar_wait(VFULL(g % kStages), (g / kStages) & 1, 200000000ull);
-            tc::mbar_wait(QFULL, 0, 1000000ull);  // (either parity: a Q copy in flight has a millisecond each)
-            tc::mbar_wait(QFULL, 1, 1000000ull);
-        }
     } else if (warp == 5) {
         // -------------------------------------------------------- MMA issuer
         constexpr uint32_t idS = tc::idesc_bf16(kRows, kKeysT, false);
@@ -571,6 +561,12 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
 
     tc::fence_before_sync();
     __syncthreads();
+    if (*abort_flag && warp == 4) {
+        tc::drain_copies(NFULL(0), kStages);
+        tc::drain_copies(VFULL(0), kStages);
+        tc::drain_copies(QFULL, 1);
+        tc::drain_copies(STAGE(0), 4);
+    }
     if (warp == 0) {
         tc::fence_after_sync();
         tc::tmem_dealloc(tmem, kTmemCols);

@@ -74,6 +74,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
         if (globaltimer_ns() - t0 > timeout_ns) return false;
     }
 }
+// For a CTA that gave up, once its warps are done: bulk copies that complete on
+// the `n` barriers from `bars` on may be in flight, and one that lands after the
+// CTA has left writes into the shared memory of a later one. Whichever parity a
+// barrier is not at returns at once; a phase in progress has a millisecond, and
+// its copies land in microseconds.
+__device__ __forceinline__ void drain_copies(uint32_t bars, int n) {
+#pragma unroll 1
+    for (int i = 0; i < 2 * n; ++i) mbar_wait(bars + 8 * (i >> 1), i & 1, 1000000ull);
+}
 // Make this thread's generic-proxy shared-memory writes visible to the async
 // proxy (TMA, tensor core).
 __device__ __forceinline__ void fence_proxy_async_smem() {
