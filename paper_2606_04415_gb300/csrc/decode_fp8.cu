@@ -29,7 +29,8 @@
 //     the softmax maximum (the row sum l takes the unscaled probabilities).
 //   * Keys past the item are masked to -inf in S and their V operands are set
 //     to zero in registers (stale slots may hold NaN codes).
-// Every mbarrier wait is bounded and raises the plan's error flag on timeout.
+// Every mbarrier wait is bounded; a timeout raises the plan's error flag, and
+// the CTA lets its copies land and exits.
 #include <cuda_fp16.h>
 #include <math.h>
 
@@ -425,6 +426,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     }
 
     __syncthreads();
+    if (*abort_flag && warp == kWarps) tc::drain_copies(FULL(0), kStages);
     if (tid == 0) {  // the last CTA out resets the work queue for the next run
         __threadfence();
         if (atomicAdd(sched + 1, 1) == static_cast<int>(gridDim.x) - 1) {

@@ -47,7 +47,8 @@
 //     the last split instead took one dependent round trip per two splits and
 //     capped the splits per sequence, and with few splits the items were too
 //     coarse to share the bandwidth evenly among the CTAs.
-// Every mbarrier wait is bounded and raises the plan's error flag on timeout.
+// Every mbarrier wait is bounded; a timeout raises the plan's error flag, and
+// the CTA lets its copies land and exits.
 //
 // The allocation-free decode (fnpu_decode_attn_noalloc) runs the same kernel
 // without a plan (kNoPlan): item i is split i / (sequences x head groups) of
@@ -495,6 +496,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     }
 
     __syncthreads();
+    if (*abort_flag && warp == kWarps) tc::drain_copies(FULL(0), kStages);
     if (!kNoPlan && tid == 0) {  // the last CTA out resets the work queue for the next run
         __threadfence();
         if (atomicAdd(sched + 1, 1) == static_cast<int>(gridDim.x) - 1) {

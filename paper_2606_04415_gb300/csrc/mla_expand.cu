@@ -36,7 +36,7 @@
 // flight cover less of the latency than these CTAs' 192, and stores add 14 us to
 // its 27.
 // Every mbarrier wait is bounded; a timeout raises bit 2 of the library-wide
-// device error flag (fnpu_check: FNPU_EDEVICE_TIMEOUT) and the CTA drains its
+// device error flag (fnpu_check: FNPU_EDEVICE_TIMEOUT) and the CTA drains its copies and
 // tensor-core work, frees its tensor memory and exits.
 #include "common.cuh"
 #include "tc.cuh"
@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kGThreads, 2)
     }
     tc::fence_before_sync();
     __syncthreads();
+    if (*abort_flag && warp == 0) tc::drain_copies(FULL(0), kGStages);
     if (warp == 1) {
         tc::fence_after_sync();
         tc::tmem_dealloc(tmem, 256);

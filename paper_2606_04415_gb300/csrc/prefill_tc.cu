@@ -45,8 +45,8 @@
 // TMEM (512 columns): S0 at 0, S1 at 128 (fp32, P over their first 64
 // columns); O0 at 256, O1 at 384.
 // Every mbarrier wait is bounded; a timeout raises the plan's error flag and
-// the CTA drains its tensor-core work, frees its tensor memory and exits.
-// Launched as a programmatic dependent of the kernel before it (the step's
+// the CTA drains its tensor-core work and copies, frees its tensor memory and
+// exits. Launched as a programmatic dependent of the kernel before it (the step's
 // KV append), the grid sets up while that kernel drains; the two loader
 // warps wait for it (griddepcontrol.wait) before their first read, and every
 // other warp reads global memory only after them. Optionally (a cooperative
@@ -840,6 +840,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     tc::fence_before_sync();
     __syncthreads();
+    if (*abort_flag && warp == 8) {
+        tc::drain_copies(KFULL(0), kKStages);
+        tc::drain_copies(VFULL(0), kVStages);
+        tc::drain_copies(QFULL, 1);
+    }
     if (warp == 0) {
         tc::fence_after_sync();
         tc::tmem_dealloc(tmem, kTmemCols);
