@@ -811,12 +811,28 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
             it.blk[i] = block_table[static_cast<int64_t>(s) * block_table_stride + kb / bs + i];
         return it;
     };
+    int64_t dec_keys = 0, num_dec = 0;
+    for (int32_t s = 0; s < num_seqs; ++s)
+        if (decode_queue(s)) {
+            dec_keys += context_len[s];
+            ++num_dec;
+        }
+    if (pl->use_dt && desc->num_kv_heads <= 2 && desc->head_dim_qk == 64 && o.decode_share_pct == 0 &&
+        !(o.flags & FNPU_PLAN_GREEN_CONTEXTS)) {
+        // One or two 64-wide kv heads leave three or two of the TMA kernel's four
+        // compute warps idle. It is the faster one while a step is light (20 of
+        // 300..8000 keys, one head: 17.8 us a step, 23.6 with the per-head kernel;
+        // 100 of 2000 23.8, 25.6), but not for many keys (140 of 2000 38.6, 28.1)
+        // or sequences (200 of 530 19.9, 18.7; 800 of 550 49.2, 33.7), and with
+        // two heads not for many sequences of several hundred keys (400 of 1100
+        // 54.5, 51.8; 800 of 550 56.1, 50.2; but 1600 of 176 39.9, 44.4).
+        pl->use_dt = desc->num_kv_heads == 1 ? num_dec <= sms && dec_keys <= 1400LL * sms
+                                             : num_dec < 2LL * sms || dec_keys < 256 * num_dec;
+    }
     // items per key range: one per group of kv heads (TMA kernel), one per kv head
     const int32_t hpi = pl->use_dt ? decode_tma_heads_per_item() : 1;
     const int32_t hgroups = (desc->num_kv_heads + hpi - 1) / hpi;
-    int64_t dec_keys = 0;
-    for (int32_t s = 0; s < num_seqs; ++s)
-        if (decode_queue(s)) dec_keys += static_cast<int64_t>(context_len[s]) * hgroups;
+    dec_keys *= hgroups;
     int32_t split = std::min(o.decode_split_keys, 1 << 30);  // (room to round up)
     if (split == 0) {
         const int64_t target = (pl->use_dt ? 2LL : 6LL) * sms;
@@ -839,6 +855,19 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
                     longest = std::max(longest, context_len[s]);
                 }
             if (items <= 2LL * sms && longest <= 32 * 64) split = 64;
+        } else if (pl->use_dt && split > 320 && desc->num_kv_heads != 4 && num_dec < 3LL * sms &&
+                   std::min(hpi, desc->num_kv_heads) * desc->head_dim_qk < 4 * 128) {
+            // Items with fewer bytes a key than four 128-wide heads are bound by
+            // their chain of stages, not by HBM: at most 512 keys, and 320 where
+            // that would be between one and two waves of items (4/2 64-wide heads,
+            // 110 of 338..8271: 60.5 us with 1536, 62.1 with 768, 50.3 with 512
+            // (934 items); 140 of 2000: 45.8 with 512 (613 items), 36.7 with 320).
+            // Four heads keep the lengths that they were tuned with.
+            split = std::min(split, 512);
+            int64_t items = 0;
+            for (int32_t s = 0; s < num_seqs; ++s)
+                if (decode_queue(s)) items += static_cast<int64_t>((context_len[s] + split - 1) / split) * hgroups;
+            if (items > 3LL * sms && items < 6LL * sms) split = 320;
         }
     }
 

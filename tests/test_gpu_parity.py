@@ -840,3 +840,29 @@ def test_mla_many_items_of_one_tile():
         assert np.array_equal(out, out2) and np.array_equal(lse, lse2)
     import paper_2606_04415_gb300 as fnpu
     assert fnpu.plan_check(st.plan) == fnpu.FNPU_OK
+
+
+@pytest.mark.parametrize("hkv,n,ctx,tma", [(1, 12, 1390, True), (1, 12, 1410, False), (1, 13, 300, False), (2, 23, 400, True),
+                                           (2, 24, 400, False), (2, 24, 255, True), (2, 24, 256, False)])
+def test_narrow_heads_change_kernels_with_the_batch(hkv, n, ctx, tma):
+    """One or two 64-wide kv heads on 12 SMs: light steps on the TMA kernel (its
+    items hold both heads), many keys or sequences on the per-head kernel, which
+    merges its own splits (one launch)."""
+    sh = W.Shape(4, hkv, 64, 64, 16, False)
+    batch = W.build_batch(sh, [1] * n, [ctx] * n, [1] * n, np.random.default_rng(n + ctx), name="narrow")
+    st = _step(batch, sms=12, split=128)
+    per = (ctx + 127) // 128
+    assert st.plan.info()["decode_items"] == n * per * (1 if tma else hkv)
+    assert st.plan.info()["launches_per_run"] == (2 if tma else 1)
+    _compare(batch, *st.results())
+
+
+@pytest.mark.parametrize("n,items", [(3, 3 * 6 * 2), (5, 5 * 10 * 2), (20, 20 * 6 * 2)])
+def test_narrow_items_are_short(n, items):
+    """Eight 64-wide kv heads on 12 SMs (36 CTAs): items of 512 keys in one wave or
+    from two waves on, of 320 between."""
+    sh = W.Shape(16, 8, 64, 64, 32, False)
+    batch = W.build_batch(sh, [1] * n, [3000] * n, [1] * n, np.random.default_rng(n), name="narrow_items")
+    st = _step(batch, sms=12)
+    assert st.plan.info()["decode_items"] == items
+    _compare(batch, *st.results())
