@@ -370,11 +370,19 @@ extern "C" int fnpu_decode_attn_noalloc(const fnpu_attn_desc *desc, int32_t num_
     rc = global_error_address(&err);
     if (rc != FNPU_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (decode_tma_supported(D, D, Hkv, G, desc->block_size)) {
-        int dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return FNPU_ECUDA;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return FNPU_ECUDA;
+    // One or two 64-wide kv heads leave three or two of the TMA kernel's four
+    // compute warps idle: few sequences end sooner on it all the same, many, or
+    // with two heads many of several hundred keys, on the kernel above (one head:
+    // 140 of 1500..2500 keys 39.4 us a call, 37.9 there; 400 of 200..2000 63.1, 44.4;
+    // two: 400 of those 68.0, 66.6; 800 of 100..1000 72.8, 71.1).
+    const bool narrow = D == 64 && (Hkv == 1   ? 4LL * num_seqs > 3LL * sms
+                                    : Hkv == 2 ? num_seqs >= 2 * sms && max_context_len >= 512
+                                               : false);
+    if (decode_tma_supported(D, D, Hkv, G, desc->block_size) && !narrow) {
         const int32_t hpi = decode_tma_heads_per_item(), hgroups = (Hkv + hpi - 1) / hpi;
         AttnParams a = {};
         a.q = q;

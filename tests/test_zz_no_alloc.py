@@ -297,3 +297,27 @@ def test_noalloc_one_call_prepares_all_later_ones():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", _ONE_CALL_PREPARES], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "prepared" in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("hkv,share,bound", [(1, 0.75, 700), (2, 2.0, 512), (2, 2.0, 511)])
+def test_noalloc_narrow_heads_on_both_sides_of_the_kernels_line(hkv, share, bound):
+    """One or two 64-wide kv heads: up to 3/4 of a sequence per SM (one head), or
+    fewer than two with bounds from 512 keys on (two heads), the TMA kernel runs,
+    beyond it the per-head one."""
+    _need_gpu()
+    import paper_2606_04415_gb300 as fnpu
+    from paper_2606_04415_gb300.step import DeviceStep
+    line = int(share * torch.cuda.get_device_properties(0).multi_processor_count)
+    for n in (line - 1, line, line + 1):
+        rng = np.random.default_rng(n)
+        ctx = rng.integers(1, bound + 1, size=n)
+        ctx[0] = bound
+        batch = W.build_batch(W.Shape(4, hkv, 64, 64, 16, False), [1] * n, ctx, [1] * n, rng, name="noalloc_narrow")
+        st = DeviceStep(batch)
+        st.append()
+        fnpu.decode_attn_noalloc(st.desc, torch.from_numpy(batch.context_len).cuda(), torch.from_numpy(batch.block_table).cuda(),
+                                 bound, st.q, st.k_cache, st.v_cache, st.out, st.lse)
+        out, lse = st.results()
+        assert fnpu.check() == fnpu.FNPU_OK
+        ref_o, ref_l = _oracle_after_append(batch)
+        assert np.abs(out - ref_o).max() <= O_TOL and np.abs(lse - ref_l).max() <= LSE_TOL
