@@ -168,3 +168,36 @@ def test_step_runs_repeatedly():
     o2, l2 = st.results()
     assert fnpu.plan_check(st.plan) == fnpu.FNPU_OK
     assert np.array_equal(o1, o2) and np.array_equal(l1, l2)
+
+
+@pytest.mark.parametrize("case", ["decode", "split decode", "one tile", "beside, 4 heads", "beside, 8 heads", "beside, fp8", "latent"])
+def test_captured_steps_replay(case):
+    """Two steps in a row, captured into a graph and replayed, give the bits of a
+    direct step: dependent launches become programmatic edges, also from one step's
+    merge or joined streams to the next step's append."""
+    import paper_2606_04415_gb300 as fnpu
+    from paper_2606_04415_gb300.step import DeviceStep
+    ql, ctx, ph = {
+        "decode": ([1] * 5, [1, 40, 17, 64, 33], [1] * 5),
+        "split decode": ([1] * 4, [900, 2500, 30, 1700], [1] * 4),
+        "one tile": ([4] * 6, [700, 1500, 3000, 521, 900, 4000], [1] * 6),
+        "latent": ([40, 1, 1], [90, 2000, 700], [0, 1, 1]),
+    }.get(case, ([600] + [1] * 20, [3000] + [150 + 190 * i for i in range(20)], [0] + [1] * 20))
+    shape = {"beside, 8 heads": W.Shape(32, 8, 128, 128, 32, False), "latent": W.SHAPES["mla"]}.get(case, W.SHAPES["qwen"])
+    batch = W.build_batch(shape, ql, ctx, ph, np.random.default_rng(5), name="captured")
+    st = DeviceStep(batch, kv_fp8="fp8" in case)
+    st.run()
+    ref = st.results()
+    if "beside" in case:
+        fnpu.plan_phase_ms(st.plan)  # (side by side)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        st.run()
+        st.run()
+    for _ in range(3):
+        st.out.fill_(float("nan"))
+        st.lse.fill_(float("nan"))
+        graph.replay()
+        got = st.results()
+        assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+    assert fnpu.plan_check(st.plan) == fnpu.FNPU_OK and fnpu.check() == fnpu.FNPU_OK
