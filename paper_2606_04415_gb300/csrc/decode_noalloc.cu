@@ -382,7 +382,7 @@ extern "C" int fnpu_decode_attn_noalloc(const fnpu_attn_desc *desc, int32_t num_
     const bool narrow = D == 64 && (Hkv == 1   ? 4LL * num_seqs > 3LL * sms
                                     : Hkv == 2 ? num_seqs >= 2 * sms && max_context_len >= 512
                                                : false);
-    if (decode_tma_supported(D, D, Hkv, G, desc->block_size) && !narrow) {
+    if (decode_tma_supported(D, D, G, desc->block_size) && !narrow) {
         const int32_t hpi = decode_tma_heads_per_item(), hgroups = (Hkv + hpi - 1) / hpi;
         AttnParams a = {};
         a.q = q;

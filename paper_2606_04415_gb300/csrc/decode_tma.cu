@@ -373,59 +373,59 @@ __global__ void __launch_bounds__(kThreads, 3)
                 const int nv = nkeys - i * kKeys;  // valid keys in this stage (>= 1)
                 const bool tail = nv < kKeys;
                 if (has_head(cur)) {  // (warp-uniform; else the warp only releases the stage)
-                if (tail) {  // zero this head's V rows past the item's keys
-                    for (int e = lane; e < (kKeys - nv) * 8 * (D / 64); e += 32) {
-                        const int hh = e / ((kKeys - nv) * 8), rem = e % ((kKeys - nv) * 8);
-                        const int sl = nv + rem / 8, ch = rem % 8;
-                        *reinterpret_cast<uint4 *>(smem + st * Cfg::kStageBytes + Cfg::kTileBytes + hh * kHalfBytes +
-                                                   (wh * kKeys + sl) * 128 + ch * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    if (tail) {  // zero this head's V rows past the item's keys
+                        for (int e = lane; e < (kKeys - nv) * 8 * (D / 64); e += 32) {
+                            const int hh = e / ((kKeys - nv) * 8), rem = e % ((kKeys - nv) * 8);
+                            const int sl = nv + rem / 8, ch = rem % 8;
+                            *reinterpret_cast<uint4 *>(smem + st * Cfg::kStageBytes + Cfg::kTileBytes + hh * kHalfBytes +
+                                                       (wh * kKeys + sl) * 128 + ch * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
-                }
-                float s[4] = {0.f, 0.f, 0.f, 0.f};
+                    float s[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                    uint32_t a0, a1, a2, a3;
-                    ldmatrix_x4(a0, a1, a2, a3, sK + dt_off(lr + 8 * (lj & 1), wh, 2 * kk + (lj >> 1)));
-                    mma_bf16_16816(s, a0, a1, a2, a3, qb[kk][0], qb[kk][1]);
-                }
-                const bool v0 = g8 < nv, v1 = g8 + 8 < nv;
-                const float x0 = v0 ? s[0] * p.scale_log2 : -INFINITY;
-                const float x1 = v0 ? s[1] * p.scale_log2 : -INFINITY;
-                const float x2 = v1 ? s[2] * p.scale_log2 : -INFINITY;
-                const float x3 = v1 ? s[3] * p.scale_log2 : -INFINITY;
-                float t0 = fmaxf(x0, x2), t1 = fmaxf(x1, x3);
-                t0 = warp_max_xor(t0, 4); t0 = warp_max_xor(t0, 8); t0 = warp_max_xor(t0, 16);
-                t1 = warp_max_xor(t1, 4); t1 = warp_max_xor(t1, 8); t1 = warp_max_xor(t1, 16);
-                const float mn0 = fmaxf(m0, t0), mn1 = fmaxf(m1, t1);
-                const float b0 = (mn0 == -INFINITY) ? 0.f : mn0;
-                const float b1 = (mn1 == -INFINITY) ? 0.f : mn1;
-                const float al0 = fast_exp2(m0 - b0), al1 = fast_exp2(m1 - b1);
-                const float p0 = fast_exp2(x0 - b0), p1 = fast_exp2(x1 - b1);
-                const float p2 = fast_exp2(x2 - b0), p3 = fast_exp2(x3 - b1);
-                l0 = l0 * al0 + p0 + p2;
-                l1 = l1 * al1 + p1 + p3;
-                m0 = mn0;
-                m1 = mn1;
+                    for (int kk = 0; kk < D / 16; ++kk) {
+                        uint32_t a0, a1, a2, a3;
+                        ldmatrix_x4(a0, a1, a2, a3, sK + dt_off(lr + 8 * (lj & 1), wh, 2 * kk + (lj >> 1)));
+                        mma_bf16_16816(s, a0, a1, a2, a3, qb[kk][0], qb[kk][1]);
+                    }
+                    const bool v0 = g8 < nv, v1 = g8 + 8 < nv;
+                    const float x0 = v0 ? s[0] * p.scale_log2 : -INFINITY;
+                    const float x1 = v0 ? s[1] * p.scale_log2 : -INFINITY;
+                    const float x2 = v1 ? s[2] * p.scale_log2 : -INFINITY;
+                    const float x3 = v1 ? s[3] * p.scale_log2 : -INFINITY;
+                    float t0 = fmaxf(x0, x2), t1 = fmaxf(x1, x3);
+                    t0 = warp_max_xor(t0, 4); t0 = warp_max_xor(t0, 8); t0 = warp_max_xor(t0, 16);
+                    t1 = warp_max_xor(t1, 4); t1 = warp_max_xor(t1, 8); t1 = warp_max_xor(t1, 16);
+                    const float mn0 = fmaxf(m0, t0), mn1 = fmaxf(m1, t1);
+                    const float b0 = (mn0 == -INFINITY) ? 0.f : mn0;
+                    const float b1 = (mn1 == -INFINITY) ? 0.f : mn1;
+                    const float al0 = fast_exp2(m0 - b0), al1 = fast_exp2(m1 - b1);
+                    const float p0 = fast_exp2(x0 - b0), p1 = fast_exp2(x1 - b1);
+                    const float p2 = fast_exp2(x2 - b0), p3 = fast_exp2(x3 - b1);
+                    l0 = l0 * al0 + p0 + p2;
+                    l1 = l1 * al1 + p1 + p3;
+                    m0 = mn0;
+                    m1 = mn1;
 #pragma unroll
-                for (int mt = 0; mt < D / 16; ++mt) {
-                    o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
-                }
-                const uint32_t r01 = pack_bf16x2(p0, p1), r23 = pack_bf16x2(p2, p3);
-                const uint32_t pb0 = movmatrix_trans(r01), pb1 = movmatrix_trans(r23);
-                uint32_t pe0 = 0u, pe1 = 0u;
-                if constexpr (kFineP) {
-                    pe0 = movmatrix_trans(bf16x2_rest(r01, p0, p1));
-                    pe1 = movmatrix_trans(bf16x2_rest(r23, p2, p3));
-                }
+                    for (int mt = 0; mt < D / 16; ++mt) {
+                        o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
+                    }
+                    const uint32_t r01 = pack_bf16x2(p0, p1), r23 = pack_bf16x2(p2, p3);
+                    const uint32_t pb0 = movmatrix_trans(r01), pb1 = movmatrix_trans(r23);
+                    uint32_t pe0 = 0u, pe1 = 0u;
+                    if constexpr (kFineP) {
+                        pe0 = movmatrix_trans(bf16x2_rest(r01, p0, p1));
+                        pe1 = movmatrix_trans(bf16x2_rest(r23, p2, p3));
+                    }
 #pragma unroll
-                for (int mt = 0; mt < D / 16; ++mt) {
-                    uint32_t a0, a1, a2, a3;
-                    ldmatrix_x4_trans(a0, a1, a2, a3, sV + dt_off(lr + 8 * (lj >> 1), wh, 2 * mt + (lj & 1)));
-                    mma_bf16_16816(o[mt], a0, a1, a2, a3, pb0, pb1);
-                    if constexpr (kFineP) mma_bf16_16816(o[mt], a0, a1, a2, a3, pe0, pe1);
-                }
-                if (tail) tc::fence_proxy_async_smem();  // order the zeroing before the next TMA write
+                    for (int mt = 0; mt < D / 16; ++mt) {
+                        uint32_t a0, a1, a2, a3;
+                        ldmatrix_x4_trans(a0, a1, a2, a3, sV + dt_off(lr + 8 * (lj >> 1), wh, 2 * mt + (lj & 1)));
+                        mma_bf16_16816(o[mt], a0, a1, a2, a3, pb0, pb1);
+                        if constexpr (kFineP) mma_bf16_16816(o[mt], a0, a1, a2, a3, pe0, pe1);
+                    }
+                    if (tail) tc::fence_proxy_async_smem();  // order the zeroing before the next TMA write
                 }
                 __syncwarp();
                 tc::mbar_arrive_warp(EMPTY(st));
@@ -703,8 +703,7 @@ int launch_merge(const AttnParams &p, cudaStream_t st) {
 
 }  // namespace
 
-bool decode_tma_supported(int d_qk, int d_v, int hkv, int group, int block_size) {
-    (void)hkv;
+bool decode_tma_supported(int d_qk, int d_v, int group, int block_size) {
     return d_qk == d_v && (d_qk == 64 || d_qk == 128) && group <= 8 && block_size % kKeys == 0;
 }
 

@@ -773,7 +773,7 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
     pl->use_mla = desc->v_in_k_latent != 0;
     pl->use_mla_tc = pl->use_mla && !(o.flags & FNPU_PLAN_NO_TCGEN05) &&
                      mla_tc_supported(desc->head_dim_qk, desc->head_dim_v, desc->num_q_heads, desc->num_kv_heads, bs);
-    pl->use_dt = !pl->use_mla && decode_tma_supported(desc->head_dim_qk, desc->head_dim_v, desc->num_kv_heads,
+    pl->use_dt = !pl->use_mla && decode_tma_supported(desc->head_dim_qk, desc->head_dim_v,
                                                       desc->num_q_heads / desc->num_kv_heads, bs);
     pl->use_tc = !pl->use_mla && !(o.flags & FNPU_PLAN_NO_TCGEN05) &&
                  prefill_tc_supported(desc->head_dim_qk, desc->head_dim_v, bs,

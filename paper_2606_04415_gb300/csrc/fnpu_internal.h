@@ -178,7 +178,7 @@ int launch_fp8_stage(const void *k_pool, const void *v_pool, const Fp8StageJob *
 bool decode_fp8_supported(int d_qk, int d_v, int hkv, int group, int block_size);
 int launch_decode_mma(const AttnParams &p, void *stream);
 int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas, bool alone);
-bool decode_tma_supported(int d_qk, int d_v, int hkv, int group, int block_size);
+bool decode_tma_supported(int d_qk, int d_v, int group, int block_size);
 int decode_tma_heads_per_item();
 // without a plan: p.na_*, num_ditems = sequences x head groups x na_max_splits,
 // num_mgroups = sequences, partial rows sequence x na_max_splits + split

@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
             int idx;
             if (!next_item(k, idx) || idx < 0) break;
             const MlaItem it = p.mitems[idx];
-            const int n = tiles_of(it), half = it.hb;
+            const int n = tiles_of(it);
             float m_run = -INFINITY, l = 0.f;
             bool ok = true;
             for (int j = 0; j < n; ++j, ++T) {
@@ -437,7 +437,6 @@ __global__ void __launch_bounds__(kThreads, 1) mla_tc_kernel(const AttnParams p,
                 tc::mbar_arrive_warp(PREADY);
             }
             if (!ok) break;
-            (void)half;
             l_buf[(k & 1) * kRows + r] = make_float2(m_run, l);
             __syncwarp();
             tc::mbar_arrive_warp(LREADY(k));
