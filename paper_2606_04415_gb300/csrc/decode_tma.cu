@@ -123,9 +123,14 @@ __device__ __forceinline__ void load_q(const AttnParams &p, int t, int head, int
     }
 }
 
-// what the bf16 pair `r` leaves of the values it was rounded from
-__device__ __forceinline__ uint32_t bf16x2_rest(uint32_t r, float lo, float hi) {
-    return pack_bf16x2(lo - __uint_as_float(r << 16), hi - __uint_as_float(r & 0xFFFF0000u));
+// A pair of probabilities as two bf16 pairs whose sum it is to 2^-16: the largest
+// bf16 values below them, and the rest. Both parts of one above zero are above
+// zero, so that an infinite V value stays infinite (rounding to nearest leaves
+// rests of zero or less, and 0 * inf or inf - inf is NaN).
+__device__ __forceinline__ void bf16x2_split(float x, float y, uint32_t &part, uint32_t &rest) {
+    const uint32_t a = max(__float_as_uint(x), 1u) - 1u, b = max(__float_as_uint(y), 1u) - 1u;
+    part = __byte_perm(a, b, 0x7632);
+    rest = pack_bf16x2(x - __uint_as_float(a & 0xFFFF0000u), y - __uint_as_float(b & 0xFFFF0000u));
 }
 
 // block ids of the item's blocks, relative block `lane` in lane `lane`
@@ -137,13 +142,13 @@ __device__ __forceinline__ int load_blk_lane(const AttnParams &p, const DtGeo &g
 
 // kRagged: the kv heads are no multiple of four, so that a warp of the last
 // group may have none (the checks cost a small step 7% where they are not needed)
-// kFineP: P enters its product as two bf16 operands, its rounding and the rest.
+// kFineP: P enters its product as two bf16 operands.
 // Where this kernel took the place of the per-head ones (without a plan, and for
 // other than four kv heads) they had a running maximum per warp and quarter of a
 // 64-key tile, so that more probabilities were exactly 1 before they were
 // rounded: 1.73e-3 off the 64-bit result without a plan (16 sequences, 32/8
 // heads) and 1.77e-3 with one (64), where one operand gives 1.81e-3 and 1.83e-3
-// and two 1.64e-3 and 1.66e-3. They cost 43.1 -> 44.7 us of that call, and a
+// and two 1.64e-3 and 1.66e-3. They cost 43.2 -> 45.0 us of that call, and a
 // light step of four kv heads, which always had one, would pay 14.3 -> 15.0.
 template <int D, bool kRagged, int kStages, bool kNoPlan, bool kFineP>
 __global__ void __launch_bounds__(kThreads, 3)
@@ -411,13 +416,18 @@ __global__ void __launch_bounds__(kThreads, 3)
                     for (int mt = 0; mt < D / 16; ++mt) {
                         o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
                     }
-                    const uint32_t r01 = pack_bf16x2(p0, p1), r23 = pack_bf16x2(p2, p3);
-                    const uint32_t pb0 = movmatrix_trans(r01), pb1 = movmatrix_trans(r23);
-                    uint32_t pe0 = 0u, pe1 = 0u;
+                    uint32_t pb0, pb1, pe0 = 0u, pe1 = 0u;
                     if constexpr (kFineP) {
-                        pe0 = movmatrix_trans(bf16x2_rest(r01, p0, p1));
-                        pe1 = movmatrix_trans(bf16x2_rest(r23, p2, p3));
+                        bf16x2_split(p0, p1, pb0, pe0);
+                        bf16x2_split(p2, p3, pb1, pe1);
+                        pe0 = movmatrix_trans(pe0);
+                        pe1 = movmatrix_trans(pe1);
+                    } else {
+                        pb0 = pack_bf16x2(p0, p1);
+                        pb1 = pack_bf16x2(p2, p3);
                     }
+                    pb0 = movmatrix_trans(pb0);
+                    pb1 = movmatrix_trans(pb1);
 #pragma unroll
                     for (int mt = 0; mt < D / 16; ++mt) {
                         uint32_t a0, a1, a2, a3;

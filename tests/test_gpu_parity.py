@@ -866,3 +866,34 @@ def test_narrow_items_are_short(n, items):
     st = _step(batch, sms=12)
     assert st.plan.info()["decode_items"] == items
     _compare(batch, *st.results())
+
+
+@pytest.mark.parametrize("hkv", [8, 4, 2])
+def test_an_infinite_value_stays_infinite(hkv):
+    """An infinite V value that a decode row sees with a probability above zero,
+    exactly 1 (a context of one key, or by far the largest score) or small, makes
+    its column infinite for the heads that share it, and nothing else; without a
+    plan as with one."""
+    import paper_2606_04415_gb300 as fnpu
+    from paper_2606_04415_gb300.step import DeviceStep
+    sh = W.Shape(4 * hkv, hkv, 128, 128, 16, False)
+    ctx = [1, 40, 40, 700]
+    batch = W.build_batch(sh, [1] * 4, ctx, [1] * 4, np.random.default_rng(hkv), name="inf_v")
+    ref_o, ref_l, _, _ = oracle.run_step(batch)
+    batch.v_new[0, 0, 3] = 0x7F80
+    for s, key in ((1, 9), (3, 333)):
+        batch.v_cache[batch.block_table[s, key // 16], key % 16, 0, 3] = 0x7F80
+    batch.v_new[2, 0, 3] = 0xFF80
+    batch.k_new[2, 0] = batch.q[2, 0]  # (the new key's score towers over the others for head 0)
+    st = DeviceStep(batch)
+    st.run()
+    outs = [st.results()]
+    fnpu.decode_attn_noalloc(st.desc, torch.from_numpy(batch.context_len).cuda(), torch.from_numpy(batch.block_table).cuda(),
+                             700, st.q, st.k_cache, st.v_cache, st.out, st.lse)
+    outs.append(st.results())
+    for out, lse in outs:
+        assert (out[[0, 1, 3], :4, 3] == np.inf).all() and (out[2, :4, 3] == -np.inf).all()
+        rest = np.ones(out.shape, bool)
+        rest[:, :4, 3] = False
+        rest[2, :4] = False  # (another key than the oracle's batch has)
+        assert np.isfinite(out[2, :4, 4:]).all() and np.abs(out - ref_o)[rest].max() <= O_TOL
