@@ -236,9 +236,11 @@ int fnpu_mixed_step(const fnpu_plan *plan, const void *k_new, const void *v_new,
 int fnpu_plan_check(const fnpu_plan *plan, void *stream);
 
 /* Synchronise `stream`, then read and clear the library-wide device error
- * flag of the current device (set by fnpu_kv_append on an out-of-range slot,
- * and by fnpu_decode_attn_noalloc on a context length or block id out of
- * range): FNPU_OK, FNPU_EDEVICE_RANGE or FNPU_ECUDA. */
+ * flag of the current device: FNPU_EDEVICE_RANGE (set by fnpu_kv_append and
+ * fnpu_mla_expand on an out-of-range slot, and by fnpu_decode_attn_noalloc on a
+ * context length or block id out of range), FNPU_EDEVICE_TIMEOUT (a bounded wait
+ * of fnpu_mla_expand or fnpu_decode_attn_noalloc gave up: the rows of that call
+ * are undefined), FNPU_OK or FNPU_ECUDA. */
 int fnpu_check(void *stream);
 
 /* Release the plan and its device workspace. Waits for the plan's stream
@@ -265,7 +267,8 @@ int fnpu_plan_info(const fnpu_plan *plan, int32_t *prefill_items, int32_t *decod
  *   Errors: FNPU_EINVAL for NULL arguments or a plan that has not run yet;
  *   FNPU_EUNSUPPORTED for a plan that does not co-locate (one phase only,
  *   latent attention, FNPU_PLAN_SEPARATE_LAUNCHES, or a number of kv heads
- *   other than four and a step that is faster with its phases in turn).
+ *   other than four and a step that is faster with its phases in turn, by the
+ *   planner's model).
  *
  * fnpu_dispatch_next_share: host arithmetic only. From the share share_pct
  * (1..99, percent of SMs, as decode_share_pct) and the phase times it gave,
@@ -315,8 +318,9 @@ int fnpu_plan_decode_share(const fnpu_plan *plan, int32_t *share_pct);
  *                 ceil(max_context_len / block_size)
  *   max_context_len  host bound on context_len; it sizes the grid
  *   split_keys    keys per split, a multiple of 64; 0 leaves it to the library
- *                 (256 or 128 for light batches where the scratch allows, else
- *                 512; requests are accepted or refused as for 512)
+ *                 (128, 256 or 512 by the number of sequences and the bound,
+ *                 where the scratch allows; requests are accepted or refused
+ *                 as for 512)
  *   q             device bf16 [num_seqs, Hq, d]; out bf16 [num_seqs, Hq, d];
  *                 lse fp32 [num_seqs, Hq]; k_cache / v_cache as above
  * Supports split K/V caches with d_qk = d_v in {64, 128} and Hq/Hkv <= 8.
@@ -338,10 +342,11 @@ int fnpu_plan_decode_share(const fnpu_plan *plan, int32_t *share_pct);
  * every kernel that a call may come to, whatever its shape and batch; make
  * that first call before any stream capture, and before device memory is full.
  * Later calls load nothing and may be captured. All calls share the one array, which keeps the
- * last call's contents; a call that merges by counters (block sizes that are
- * no multiple of 16) clears them itself with cudaMemsetAsync on `stream`. Calls that overlap on the GPU (on different
- * streams, or with no ordering between them) race on the array and must not
- * be issued.
+ * last call's contents; a call that merges by counters (block sizes that are no
+ * multiple of 16, and many sequences of one or two 64-wide kv heads) clears them
+ * itself with cudaMemsetAsync on `stream`. Calls that overlap on the GPU (on
+ * different streams, or with no ordering between them) race on the array and must
+ * not be issued.
  */
 #define FNPU_NOALLOC_SCRATCH_BYTES (16u << 20)
 int fnpu_decode_attn_noalloc(const fnpu_attn_desc *desc, int32_t num_seqs,

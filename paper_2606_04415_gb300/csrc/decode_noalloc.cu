@@ -10,8 +10,9 @@
 //
 // With block sizes that are multiples of 16 the TMA-fed decode kernel and its
 // merge run without a plan (decode_tma.cu; 16 decodes of 200..6000 keys, 32
-// query and 8 kv heads: 43.1 us a call against 80.0 with the kernel below);
-// other block sizes take the kernel below:
+// query and 8 kv heads: 45.0 us a call against 80.1 with the kernel below);
+// other block sizes, and many sequences of one or two 64-wide kv heads, take the
+// kernel below:
 //
 //   * the work list is implicit: CTA b handles split b % max_splits of
 //     (sequence, kv head) b / max_splits, reading the context length on the
@@ -406,12 +407,12 @@ extern "C" int fnpu_decode_attn_noalloc(const fnpu_attn_desc *desc, int32_t num_
         // The split length where the caller leaves it open (0: requests are
         // judged at 512 keys): shorter ones while the items that the host's
         // bound allows are at most two per SM, so that a light batch ends
-        // sooner (one sequence of up to 6000 keys 15.2 us a call with 128
-        // keys, 27.1 with 512; 8 of up to 4000 with two head groups 18.8 with
-        // 256, 27.5 with 512; but 32 of up to 4000, 512 items of 256 keys,
-        // 40.9 against 33.2 with 512), and 256 where 512 would give CTAs
-        // unequal numbers of items (32 of up to 4000 with two head groups 54.0
-        // against 64.1); always within the scratch.
+        // sooner (one sequence of 6000 keys 16.8 us with its append with 128
+        // keys, 31.3 with 512; 8 of up to 4000 with two head groups 21.5 with
+        // 256, 31.4 with 512; but 32 of up to 4000, 512 items of 256 keys,
+        // 43.8 against 37.1 with 512), and 256 where 512 would give CTAs
+        // unequal numbers of items (32 of up to 4000 with two head groups 66.4
+        // against 67.3); always within the scratch.
         auto items = [&](int32_t sk) {
             return static_cast<int64_t>(num_seqs) * hgroups * ((max_context_len + sk - 1) / sk);
         };

@@ -2,8 +2,8 @@
 // (d = 64 or 128, G <= 8 query heads per kv head, block size a multiple of
 // 16). An item covers up to four kv heads of its keys; with more than four,
 // the heads go in groups of four, each an item of its own. (For 32 query and
-// 8 kv heads, a 1024-token chunk beside 64 decodes: 140.0 us with the per-head
-// cp.async kernel ahead of the prefill, whose decode streams 2.8 TB/s; 90.4
+// 8 kv heads, a 1024-token chunk beside 64 decodes: 140.3 us with the per-head
+// cp.async kernel ahead of the prefill, whose decode streams 2.8 TB/s; 91.6
 // us with this one beside the prefill.)
 //
 // Decode is bound by KV-cache reads (Sec. 1, Sec. 3.3, Fig. 2). The kernel is
@@ -654,7 +654,7 @@ int launch_dt(const AttnParams &p, cudaStream_t st, int grid, bool after_prev) {
 // The ring depth: an SM's shared memory holds six 32 KB stages (d = 128; twelve
 // for d = 64), and all of them should be in flight whatever the number of CTAs on
 // it (d = 64, 2 kv heads, 64 decodes of 500..4000 keys: 28.2 us a step with half
-// of them, 24.3 with all).
+// of them, 24.3 with all; 25.9 since P goes in as two operands).
 template <int D, bool kRagged, bool kNoPlan, bool kFineP>
 int launch_dt(const AttnParams &p, cudaStream_t st, int max_ctas, bool alone) {
     const int grid = p.num_ditems < max_ctas ? p.num_ditems : max_ctas;

@@ -201,7 +201,9 @@ constexpr int64_t kTcDualMergeCost = 1;
 // A chunk of at most one Q tile takes two key tiles a step from this many on
 // (the exchange of the two paths costs about one tile). The short last item of a
 // longer chunk does not: beside full items it is over early either way, and four
-// chunks of 512 tokens took 39.7 us with it against 34.5.
+// chunks of 512 tokens took 39.7 us with it against 34.5. (The kernel needs a key
+// tile on each path: pieces of such a unit have two steps or more, as no cap on
+// them is below four.)
 constexpr int32_t kDualTiles = 4;
 
 // First tile of split j of n over ntiles tiles (split n is the end).
@@ -676,7 +678,8 @@ int fnpu_check(void *stream) {
     int flag = 0;
     const int rc = read_and_clear_global_error(stream, &flag);
     if (rc != FNPU_OK) return rc;
-    if (flag & 4) return FNPU_EDEVICE_TIMEOUT;  // a bounded wait of the MLA expansion gave up
+    // bit 2: a bounded wait of the MLA expansion or the allocation-free decode gave up
+    if (flag & 4) return FNPU_EDEVICE_TIMEOUT;
     return flag ? FNPU_EDEVICE_RANGE : FNPU_OK;
 }
 
@@ -1040,7 +1043,8 @@ int plan_fill(fnpu_plan *pl, const fnpu_attn_desc *desc, int32_t num_seqs, const
         // decodes: 33.4, 29.5; below, 9.8 MB and 6 us: 23.9, 26.3), of 25 us
         // where they do not (219 x 3 tokens on 5223: 78.9, 58.2; but 1603 tokens
         // on 2 and 35 short decodes, 22.5 us by the model: 42.2, 47.5). Four kv
-        // heads co-locate always: such plans report phase times.
+        // heads co-locate always: callers of such plans have always been able to
+        // read their phase times and share, and a status does not depend on lengths.
         const double span = static_cast<double>(lpt_makespan(cost_histogram(item_tiles), sms)) * tile_scale * kTileSec;
         const bool wide = 4 * static_cast<int64_t>(tc_units.size()) > 3 * static_cast<int64_t>(sms);
         pl->coloc = span >= (dec_bytes >= 20e-6 * kDecodeAllBps ? 5e-6 : wide ? 25e-6 : 8e-6);

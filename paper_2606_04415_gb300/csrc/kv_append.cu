@@ -16,8 +16,10 @@ namespace fnpu {
 
 // Library-wide device error flag, one per device that loads the library;
 // read and cleared by fnpu_check(). Bit 0: an append met an out-of-range
-// slot; bit 1: the allocation-free decode met a context length or a block
-// id out of range.
+// slot, or the MLA expansion's gather one; bit 1: the allocation-free decode
+// met a context length or a block id out of range; bit 2: a bounded wait of the
+// MLA expansion or of the allocation-free decode gave up, or a kernel of theirs
+// found its shared memory misaligned.
 __device__ int g_device_error = 0;
 
 __global__ void __launch_bounds__(256) kv_append_kernel(

@@ -376,8 +376,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // issuer's 15 KB a step and the softmax evicted each other from the
         // instruction cache. With that, one place in the code per product and
         // one box per producer lane, the step of 2048 tokens on a prefix of
-        // 7000 beside 128 decodes takes 197 us (205 before), four 512-token
-        // chunks 34.5 (39.1).
+        // 7000 beside 128 decodes takes 207.5 us (212.7 before, both on one box),
+        // four 512-token chunks 35.7 (39.5), a 1024-token chunk of 192-wide keys
+        // with its expansion 111.6 (118.6).
         constexpr uint32_t idS = F16 ? tc::idesc_f16(kRows, kKeys, false) : tc::idesc_bf16(kRows, kKeys, false);
         constexpr uint32_t idO = F16 ? tc::idesc_f16(kRows, DV, true) : tc::idesc_bf16(kRows, DV, true);
         const uint32_t utmem = __shfl_sync(0xffffffffu, tmem, 0);
