@@ -727,6 +727,7 @@ int launch_decode_tma(const AttnParams &p, void *stream, int max_ctas, bool alon
 }
 
 int prepare_decode_tma_noplan() {
+    (void)tensor_map_encoder();  // (looked up once; a launch reports it if there is none)
     const int rc = prepare_noplan<64>();
     return rc != FNPU_OK ? rc : prepare_noplan<128>();
 }

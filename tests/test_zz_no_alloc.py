@@ -256,7 +256,7 @@ def call(n, ctx, hq, hkv, d, bs=16):
     out, lse = torch.empty_like(q), torch.empty(n, hq, device="cuda")
     return (lambda: fnpu.decode_attn_noalloc(desc, cl, bt, ctx, q, k, v, out, lse)), out, lse
 
-small = call(1, 16, 4, 2, 64)
+small = call(1, 16, 4, 2, 64, 24)
 others = [call(n, ctx, hq, hkv, d, bs) for hq, hkv, d, bs in
           [(32, 8, 128, 16), (9, 3, 128, 16), (4, 4, 64, 16), (6, 2, 64, 16), (28, 4, 128, 24), (4, 4, 64, 24)]
           for n, ctx in [(1, 60), (1, 5000), (20, 2000), (60, 4000)]]
