@@ -70,8 +70,8 @@ def test_noalloc_decode_matches_oracle_and_planned_path_twice(split_keys):
 def test_noalloc_decode_d64_partial_group_single_and_multi_split():
     """head_dim 64 with 3 query heads per kv head (the 8 MMA columns only
     partly filled); contexts from 1 key up to and past one split, so that
-    single-split sequences (written directly, no counters) and split ones
-    (merged by the last split) both occur, checked against the oracle and the
+    single-split sequences (written directly) and split ones (merged from their
+    partials) both occur, checked against the oracle and the
     planned path on two calls in a row."""
     _need_gpu()
     import paper_2606_04415_gb300 as fnpu
